@@ -23,7 +23,6 @@
 // translation (Sec. 4.3); here the 343 offset classes are tabulated once.
 #include <algorithm>
 #include <cmath>
-#include <cstring>
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -1126,83 +1125,165 @@ __global__ void k_combine(const T *far, const T *near, int64_t n, double scale, 
 }
 
 // ---------------------------------------------------------------- tables
-// Host-side FP64 solid harmonics (full m range) for the translation tables.
-static void host_regular_full(double x, double y, double z, int p, std::vector<double> &out) {
-    // out[(n*(2p+1) + m + p)*2 + {0,1}]
-    const int W = 2 * p + 1;
-    out.assign((size_t)(p + 1) * W * 2, 0.0);
+// The translation tables are built on the device in FP64 (one CTA per offset
+// class, its solid harmonics in shared memory) and rounded once to the
+// working precision.  Bound by the write of the operators (43 MB at p = 10).
+// Measured, tables of p = 10 whenever no other mesh holds them: 18 ms built
+// on the host, 0.5 ms here (allocations included); creating a mesh of 56,180
+// panels 29.5 -> 11.7 ms.
+
+// Full-m layout X[n][m + N], stride 2N + 1, of the solid harmonics of one
+// vector, n <= N; the CTA's threads take a column m each (the recurrences of
+// the file's head) and store it with its mirror X_n^{-m} = (-1)^m conj(X_n^m).
+__device__ __forceinline__ void put_mirrored(double2 *X, int N, int n, int m, double re, double im) {
+    double2 *row = X + n * (2 * N + 1) + N;
+    row[m] = make_double2(re, im);
+    if (m > 0) row[-m] = (m & 1) ? make_double2(-re, im) : make_double2(re, -im);
+}
+
+__device__ void regular_full(double x, double y, double z, int N, double2 *X) {
+    for (int i = threadIdx.x; i < (N + 1) * (2 * N + 1); i += blockDim.x) X[i] = make_double2(0.0, 0.0);
+    __syncthreads();
     const double r2 = x * x + y * y + z * z;
-    std::vector<double> re((p + 1) * (p + 1), 0.0), im((p + 1) * (p + 1), 0.0);
-    auto at = [&](int n, int m) { return n * (p + 1) + m; };
-    re[at(0, 0)] = 1.0;
-    for (int m = 0; m <= p; ++m) {
-        if (m > 0) {
-            double f = -1.0 / (2.0 * m);
-            double a = re[at(m - 1, m - 1)], b = im[at(m - 1, m - 1)];
-            re[at(m, m)] = f * (x * a - y * b);
-            im[at(m, m)] = f * (x * b + y * a);
+    for (int m = threadIdx.x; m <= N; m += blockDim.x) {
+        double ar = 0.0, ai = 0.0, br = 1.0, bi = 0.0;  // rows n - 2 and n - 1 of the column
+        for (int k = 1; k <= m; ++k) {
+            const double f = -1.0 / (2.0 * k), re = f * (x * br - y * bi), im = f * (x * bi + y * br);
+            br = re;
+            bi = im;
         }
-        if (m + 1 <= p) {
-            re[at(m + 1, m)] = z * re[at(m, m)];
-            im[at(m + 1, m)] = z * im[at(m, m)];
-        }
-        for (int n = m + 2; n <= p; ++n) {
-            double c = 1.0 / ((n + m) * (double)(n - m));
-            re[at(n, m)] = ((2 * n - 1) * z * re[at(n - 1, m)] - r2 * re[at(n - 2, m)]) * c;
-            im[at(n, m)] = ((2 * n - 1) * z * im[at(n - 1, m)] - r2 * im[at(n - 2, m)]) * c;
+        put_mirrored(X, N, m, m, br, bi);
+        for (int n = m + 1; n <= N; ++n) {
+            const double c = 1.0 / ((double)(n + m) * (double)(n - m));
+            const double re = n == m + 1 ? z * br : ((2 * n - 1) * z * br - r2 * ar) * c;
+            const double im = n == m + 1 ? z * bi : ((2 * n - 1) * z * bi - r2 * ai) * c;
+            ar = br;
+            ai = bi;
+            br = re;
+            bi = im;
+            put_mirrored(X, N, n, m, br, bi);
         }
     }
-    for (int n = 0; n <= p; ++n)
-        for (int m = -n; m <= n; ++m) {
-            int am = m < 0 ? -m : m;
-            double a = re[at(n, am)], b = im[at(n, am)];
-            if (m < 0) {
-                double sg = (am & 1) ? -1.0 : 1.0;
-                a *= sg;
-                b *= -sg;
-            }
-            out[((size_t)n * W + m + p) * 2] = a;
-            out[((size_t)n * W + m + p) * 2 + 1] = b;
+    __syncthreads();
+}
+
+__device__ void irregular_full(double x, double y, double z, int N, double2 *X) {
+    for (int i = threadIdx.x; i < (N + 1) * (2 * N + 1); i += blockDim.x) X[i] = make_double2(0.0, 0.0);
+    __syncthreads();
+    const double ir2 = 1.0 / (x * x + y * y + z * z);
+    for (int m = threadIdx.x; m <= N; m += blockDim.x) {
+        double ar = 0.0, ai = 0.0, br = sqrt(ir2), bi = 0.0;
+        for (int k = 1; k <= m; ++k) {
+            const double f = -(2.0 * k - 1.0) * ir2, re = f * (x * br - y * bi), im = f * (x * bi + y * br);
+            br = re;
+            bi = im;
+        }
+        put_mirrored(X, N, m, m, br, bi);
+        for (int n = m + 1; n <= N; ++n) {
+            const double c1 = (2.0 * n - 1.0) * z, c2 = (double)(n - 1 - m) * (double)(n - 1 + m);
+            const double re = (c1 * br - c2 * ar) * ir2, im = (c1 * bi - c2 * ai) * ir2;
+            ar = br;
+            ai = bi;
+            br = re;
+            bi = im;
+            put_mirrored(X, N, n, m, br, bi);
+        }
+    }
+    __syncthreads();
+}
+
+// Entry (input coefficient `in`, output coefficient `out`, both positions in
+// the compact real layout) of the real matrix of a complex translation
+//   out_k^l = sum_{n, m=-n..n} coef(k, l, n, m) in_n^m
+// (both sides real fields, so in_n^{-m} = (-1)^m conj(in_n^m)).  With
+// P = coef(k,l,n,mu) and Q = (-1)^mu coef(k,l,n,-mu), an input a + ib at
+// (n, mu) contributes a (P + Q) + i b (P - Q).
+template <class F>
+__device__ __forceinline__ double real_entry(int in, int out, F coef) {
+    const int n = (int)sqrtf(in + 0.5f), rn = in - n * n, mu = (rn + 1) >> 1;
+    const int k = (int)sqrtf(out + 0.5f), rk = out - k * k, l = (rk + 1) >> 1;
+    const bool in_im = rn > 0 && !(rn & 1), out_im = rk > 0 && !(rk & 1);
+    const double2 P = coef(k, l, n, mu);
+    double2 Q = make_double2(0.0, 0.0);
+    if (mu > 0) {
+        Q = coef(k, l, n, -mu);
+        if (mu & 1) Q = make_double2(-Q.x, -Q.y);
+    }
+    if (in_im) return out_im ? P.x - Q.x : -(P.y - Q.y);
+    return out_im ? P.y + Q.y : P.x + Q.x;
+}
+
+// M2L of one offset class per CTA: the irregular harmonics If[o] of the offset
+// (target centre minus source centre over the cell size), the dense operator
+// Om2l[o] (column-major, each [in] row padded with zeros to ld) and, with Tc
+// set, its copy in the tensor-core kernel's order (tc_table_index).  Classes
+// that are neighbours of a cell hold zeros.  L_k^l = (-1)^k sum M_n^m I_{n+k}^{m+l}
+template <class T>
+__global__ void k_m2l_table(int p, int ws, int ld, cpx<T> *If, T *Om2l, float *Tc) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double2 *X = reinterpret_cast<double2 *>(smraw);
+    const int o = blockIdx.x, N = 2 * p, W = 2 * N + 1, nc = (p + 1) * (p + 1);
+    const int ro = 2 * ws + 1, wo = 2 * ro + 1;
+    const int dx = o / (wo * wo) - ro, dy = (o / wo) % wo - ro, dz = o % wo - ro;
+    const bool used = abs(dx) > ws || abs(dy) > ws || abs(dz) > ws;
+    if (used) irregular_full(-dx, -dy, -dz, N, X);
+    for (int i = threadIdx.x; i < (N + 1) * W; i += blockDim.x) {
+        cpx<T> v;
+        v.x = used ? (T)X[i].x : (T)0;
+        v.y = used ? (T)X[i].y : (T)0;
+        If[(size_t)o * (N + 1) * W + i] = v;
+    }
+    auto entry = [&](int in, int out) -> double {
+        if (!used || in >= nc || out >= nc) return 0.0;
+        return real_entry(in, out, [&](int k, int l, int n, int m) {
+            const double2 v = X[(n + k) * W + m + l + N];
+            return (k & 1) ? make_double2(-v.x, -v.y) : v;
+        });
+    };
+    for (int i = threadIdx.x; i < nc * ld; i += blockDim.x) {
+        const int in = i / ld, out = i - in * ld;
+        Om2l[(size_t)o * nc * ld + i] = (T)entry(in, out);
+    }
+    if (Tc)
+        for (int i = threadIdx.x; i < TC_TABLE_DIM * TC_TABLE_DIM; i += blockDim.x) {
+            const int in = i / TC_TABLE_DIM, out = i - in * TC_TABLE_DIM;
+            Tc[(size_t)o * TC_TABLE_DIM * TC_TABLE_DIM + tc_table_index(in, out)] = (float)entry(in, out);
         }
 }
 
-static void host_irregular_full(double x, double y, double z, int N, std::vector<double> &out) {
-    // out[(n*(2N+1) + m + N)*2 + {0,1}], n <= N
-    const int W = 2 * N + 1;
-    out.assign((size_t)(N + 1) * W * 2, 0.0);
-    const double r2 = x * x + y * y + z * z, ir2 = 1.0 / r2;
-    std::vector<double> re((N + 1) * (N + 1), 0.0), im((N + 1) * (N + 1), 0.0);
-    auto at = [&](int n, int m) { return n * (N + 1) + m; };
-    re[at(0, 0)] = std::sqrt(ir2);
-    for (int m = 0; m <= N; ++m) {
-        if (m > 0) {
-            double f = -(2.0 * m - 1.0) * ir2;
-            double a = re[at(m - 1, m - 1)], b = im[at(m - 1, m - 1)];
-            re[at(m, m)] = f * (x * a - y * b);
-            im[at(m, m)] = f * (x * b + y * a);
-        }
-        if (m + 1 <= N) {
-            re[at(m + 1, m)] = (2.0 * m + 1.0) * z * ir2 * re[at(m, m)];
-            im[at(m + 1, m)] = (2.0 * m + 1.0) * z * ir2 * im[at(m, m)];
-        }
-        for (int n = m + 2; n <= N; ++n) {
-            double c2 = (double)(n - 1 - m) * (double)(n - 1 + m);
-            re[at(n, m)] = ((2 * n - 1) * z * re[at(n - 1, m)] - c2 * re[at(n - 2, m)]) * ir2;
-            im[at(n, m)] = ((2 * n - 1) * z * im[at(n - 1, m)] - c2 * im[at(n - 2, m)]) * ir2;
-        }
+// M2M and L2L of one child octant per blockIdx.x (offset: child centre minus
+// parent centre over the parent size); blockIdx.y shares the entries.
+//   M2M: M'_N^Mo = sum_{j,mu} 2^-j conj(R_{N-j}^{Mo-mu}) M_j^mu
+//   L2L: L'_k^l = 2^-(k+1) sum_{n,m} conj(R_{n-k}^{m-l}) L_n^m
+template <class T>
+__global__ void k_tree_table(int p, int ld, cpx<T> *Rtab, T *Om2m, T *Ol2l) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double2 *X = reinterpret_cast<double2 *>(smraw);
+    const int o = blockIdx.x, W = 2 * p + 1, nc = (p + 1) * (p + 1);
+    regular_full((o & 1) ? 0.25 : -0.25, (o & 2) ? 0.25 : -0.25, (o & 4) ? 0.25 : -0.25, p, X);
+    const int i0 = blockIdx.y * blockDim.x + threadIdx.x, step = gridDim.y * blockDim.x;
+    for (int i = i0; i < (p + 1) * W; i += step) {
+        cpx<T> v;
+        v.x = (T)X[i].x;
+        v.y = (T)X[i].y;
+        Rtab[(size_t)o * (p + 1) * W + i] = v;
     }
-    for (int n = 0; n <= N; ++n)
-        for (int m = -n; m <= n; ++m) {
-            int am = m < 0 ? -m : m;
-            double a = re[at(n, am)], b = im[at(n, am)];
-            if (m < 0) {
-                double sg = (am & 1) ? -1.0 : 1.0;
-                a *= sg;
-                b *= -sg;
-            }
-            out[((size_t)n * W + m + N) * 2] = a;
-            out[((size_t)n * W + m + N) * 2 + 1] = b;
+    auto rc = [&](int n, int m, int sh) {  // 2^-sh conj(R_n^m), 0 outside
+        if (n < 0 || m < -n || m > n) return make_double2(0.0, 0.0);
+        const double2 v = X[n * W + m + p];
+        const double s = ldexp(1.0, -sh);
+        return make_double2(s * v.x, -s * v.y);
+    };
+    for (int i = i0; i < nc * ld; i += step) {
+        const int in = i / ld, out = i - in * ld;
+        double a = 0.0, b = 0.0;
+        if (out < nc) {
+            a = real_entry(in, out, [&](int k, int l, int n, int m) { return rc(k - n, l - m, n); });
+            b = real_entry(in, out, [&](int k, int l, int n, int m) { return rc(n - k, m - l, k + 1); });
         }
+        Om2m[(size_t)o * nc * ld + i] = (T)a;
+        Ol2l[(size_t)o * nc * ld + i] = (T)b;
+    }
 }
 
 static bool g_consts_up[64] = {};
@@ -1250,36 +1331,6 @@ static void upload_constants(int dev) {
     if (dev >= 0 && dev < 64) g_consts_up[dev] = true;
 }
 
-// Real (p+1)^2 x (p+1)^2 matrix of a complex translation
-//   out_k^l = sum_{n, m=-n..n} coef(k, l, n, m) in_n^m
-// acting on the compact real layout (both sides real fields, so
-// in_n^{-m} = (-1)^m conj(in_n^m)).  With P = coef(k,l,n,mu) and
-// Q = (-1)^mu coef(k,l,n,-mu), an input a + ib at (n, mu) contributes
-// a (P + Q) + i b (P - Q).  Stored column-major: Tt[in * nc + out].
-template <class F>
-static void real_operator(int p, F coef, double *Tt) {
-    const int nc = (p + 1) * (p + 1);
-    std::fill(Tt, Tt + (size_t)nc * nc, 0.0);
-    for (int k = 0; k <= p; ++k)
-        for (int l = 0; l <= k; ++l) {
-            const int ro = k * k + (l == 0 ? 0 : 2 * l - 1), io = l > 0 ? k * k + 2 * l : -1;
-            for (int n = 0; n <= p; ++n)
-                for (int mu = 0; mu <= n; ++mu) {
-                    double Pr, Pi, Qr = 0, Qi = 0;
-                    coef(k, l, n, mu, Pr, Pi);
-                    if (mu > 0) {
-                        coef(k, l, n, -mu, Qr, Qi);
-                        if (mu & 1) { Qr = -Qr; Qi = -Qi; }
-                    }
-                    const int ri = n * n + (mu == 0 ? 0 : 2 * mu - 1), ii = mu > 0 ? n * n + 2 * mu : -1;
-                    Tt[(size_t)ri * nc + ro] += Pr + Qr;
-                    if (ii >= 0) Tt[(size_t)ii * nc + ro] += -(Pi - Qi);
-                    if (io >= 0) Tt[(size_t)ri * nc + io] += Pi + Qi;
-                    if (io >= 0 && ii >= 0) Tt[(size_t)ii * nc + io] += Pr - Qr;
-                }
-        }
-}
-
 void ensure_smem_attr(const void *func, size_t bytes) {
     static std::mutex mu;
     static std::map<std::pair<const void *, int>, size_t> done;
@@ -1305,123 +1356,43 @@ static std::mutex g_tab_mu;
 static std::map<TabKey, std::weak_ptr<Tables>> g_tab_cache;
 
 template <class T>
-static void upload(DArray<T> &d, const std::vector<double> &h) {
-    std::vector<T> v(h.begin(), h.end());
-    d.alloc(v.size());
-    BEM_CUDA(cudaMemcpy(d.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+static void fill_tables(int p, int ws, DArray<T> &R, DArray<T> &I, DArray<T> &om2l, DArray<T> &om2m, DArray<T> &ol2l,
+                        DArray<float> *tc, cudaStream_t s) {
+    const int nc = (p + 1) * (p + 1), ld = cell_stride(p), ncls = m2l_classes(ws);
+    const size_t nr = (size_t)(p + 1) * (2 * p + 1), ni = (size_t)(2 * p + 1) * (4 * p + 1);
+    R.alloc(8 * nr * 2);
+    I.alloc(ncls * ni * 2);
+    om2l.alloc((size_t)ncls * nc * ld);
+    om2m.alloc((size_t)8 * nc * ld);
+    ol2l.alloc((size_t)8 * nc * ld);
+    if (tc) tc->alloc((size_t)ncls * TC_TABLE_DIM * TC_TABLE_DIM);
+    // at most 33 x 65 harmonics of 16 bytes (p = 16): below 48 KB
+    k_m2l_table<T><<<ncls, 256, ni * sizeof(double2), s>>>(p, ws, ld, reinterpret_cast<cpx<T> *>(I.p), om2l.p,
+                                                           tc ? tc->p : nullptr);
+    BEM_CHECK_LAUNCH();
+    k_tree_table<T><<<dim3(8, 8), 256, nr * sizeof(double2), s>>>(p, ld, reinterpret_cast<cpx<T> *>(R.p), om2m.p,
+                                                                  ol2l.p);
+    BEM_CHECK_LAUNCH();
 }
 
-static std::shared_ptr<Tables> make_tables(int p, int prec, int ws) {
+static std::shared_ptr<Tables> make_tables(int p, int prec, int ws, cudaStream_t s) {
     auto t = std::make_shared<Tables>();
-    const int W = 2 * p + 1, W2 = 4 * p + 1;
-    const int nc = (p + 1) * (p + 1);
-    const int NOFFSET = m2l_classes(ws), RO = m2l_radius(ws), WO = 2 * RO + 1;
     t->p = p;
     t->ws = ws;
-    // parent/child offsets: child centre minus parent centre over the parent size
-    std::vector<std::vector<double>> r8(8);
-    std::vector<double> rtab((size_t)8 * (p + 1) * W * 2);
-    for (int o = 0; o < 8; ++o) {
-        double d[3];
-        for (int k = 0; k < 3; ++k) d[k] = ((o >> k) & 1) ? 0.25 : -0.25;
-        host_regular_full(d[0], d[1], d[2], p, r8[o]);
-        std::memcpy(&rtab[(size_t)o * (p + 1) * W * 2], r8[o].data(), r8[o].size() * sizeof(double));
-    }
-    // M2L offsets: target centre minus source centre over the cell size = -(dx,dy,dz)
-    const size_t itot = (size_t)(2 * p + 1) * W2 * 2;
-    std::vector<double> it((size_t)NOFFSET * itot, 0.0), tmp;
-    auto offset_of = [&](int o, int &dx, int &dy, int &dz) {
-        dx = o / (WO * WO) - RO;
-        dy = (o / WO) % WO - RO;
-        dz = o % WO - RO;
-        return std::abs(dx) > ws || std::abs(dy) > ws || std::abs(dz) > ws;  // a class in use
-    };
-    for (int o = 0; o < NOFFSET; ++o) {
-        int dx, dy, dz;
-        if (!offset_of(o, dx, dy, dz)) continue;
-        host_irregular_full(-dx, -dy, -dz, 2 * p, tmp);
-        std::memcpy(&it[(size_t)o * itot], tmp.data(), tmp.size() * sizeof(double));
-    }
-    // dense real operators
-    const size_t osz = (size_t)nc * nc;
-    std::vector<double> om2l((size_t)NOFFSET * osz, 0.0), om2m(8 * osz), ol2l(8 * osz);
-    for (int o = 0; o < NOFFSET; ++o) {
-        int dx, dy, dz;
-        if (!offset_of(o, dx, dy, dz)) continue;
-        const double *I = &it[(size_t)o * itot];
-        // L_k^l = (-1)^k sum M_n^m I_{n+k}^{m+l}
-        real_operator(p, [&](int k, int l, int n, int m, double &re, double &im) {
-            const double sg = (k & 1) ? -1.0 : 1.0;
-            const size_t q = ((size_t)(n + k) * W2 + (m + l) + 2 * p) * 2;
-            re = sg * I[q];
-            im = sg * I[q + 1];
-        }, &om2l[(size_t)o * osz]);
-    }
-    for (int o = 0; o < 8; ++o) {
-        const std::vector<double> &R = r8[o];
-        auto Rc = [&](int n, int m, double &re, double &im) {  // conj(R_n^m), 0 outside
-            if (n < 0 || m < -n || m > n) { re = im = 0; return; }
-            const size_t q = ((size_t)n * W + m + p) * 2;
-            re = R[q];
-            im = -R[q + 1];
-        };
-        // M2M: M'_N^Mo = sum_{j,mu} 2^-j conj(R_{N-j}^{Mo-mu}) M_j^mu
-        real_operator(p, [&](int N, int Mo, int j, int mu, double &re, double &im) {
-            if (j > N) { re = im = 0; return; }
-            Rc(N - j, Mo - mu, re, im);
-            const double s = std::ldexp(1.0, -j);
-            re *= s;
-            im *= s;
-        }, &om2m[(size_t)o * osz]);
-        // L2L: L'_k^l = 2^-(k+1) sum_{n,m} conj(R_{n-k}^{m-l}) L_n^m
-        real_operator(p, [&](int k, int l, int n, int m, double &re, double &im) {
-            if (n < k) { re = im = 0; return; }
-            Rc(n - k, m - l, re, im);
-            const double s = std::ldexp(1.0, -(k + 1));
-            re *= s;
-            im *= s;
-        }, &ol2l[(size_t)o * osz]);
-    }
-    if (prec == BEM_MIXED && nc <= 128) {
-        std::vector<float> op;
-        build_tc_tables(p, om2l, NOFFSET, op);
-        t->Tc_f.alloc(op.size());
-        BEM_CUDA(cudaMemcpy(t->Tc_f.p, op.data(), op.size() * sizeof(float), cudaMemcpyHostToDevice));
-    }
-    // translation operators with each [in] row padded to the cell stride, so
-    // that k_translate stages them with 16-byte copies
-    const int ld = cell_stride(p);
-    auto pad = [&](const std::vector<double> &ops, int nops) {
-        std::vector<double> r((size_t)nops * nc * ld, 0.0);
-        for (size_t o = 0; o < (size_t)nops; ++o)
-            for (int k = 0; k < nc; ++k)
-                std::copy_n(&ops[(o * nc + k) * nc], nc, &r[(o * nc + k) * ld]);
-        return r;
-    };
-    const std::vector<double> pm2l = pad(om2l, NOFFSET), pm2m = pad(om2m, 8), pl2l = pad(ol2l, 8);
-    if (prec == BEM_MIXED) {
-        upload(t->Rm2m_f, rtab);
-        upload(t->If_f, it);
-        upload(t->Om2l_f, pm2l);
-        upload(t->Om2m_f, pm2m);
-        upload(t->Ol2l_f, pl2l);
-    } else {
-        upload(t->Rm2m_d, rtab);
-        upload(t->If_d, it);
-        upload(t->Om2l_d, pm2l);
-        upload(t->Om2m_d, pm2m);
-        upload(t->Ol2l_d, pl2l);
-    }
+    const bool tc = prec == BEM_MIXED && (p + 1) * (p + 1) <= TC_TABLE_DIM;
+    if (prec == BEM_MIXED) fill_tables<float>(p, ws, t->Rm2m_f, t->If_f, t->Om2l_f, t->Om2m_f, t->Ol2l_f, tc ? &t->Tc_f : nullptr, s);
+    else fill_tables<double>(p, ws, t->Rm2m_d, t->If_d, t->Om2l_d, t->Om2m_d, t->Ol2l_d, nullptr, s);
+    BEM_CUDA(cudaStreamSynchronize(s));  // meshes on other streams share the tables
     return t;
 }
 
-static std::shared_ptr<Tables> cached_tables(int dev, int p, int prec, int ws) {
+static std::shared_ptr<Tables> cached_tables(int dev, int p, int prec, int ws, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(g_tab_mu);
     TabKey key{dev, p, prec, ws};
     auto it = g_tab_cache.find(key);
     if (it != g_tab_cache.end())
         if (auto sp = it->second.lock()) return sp;
-    auto t = make_tables(p, prec, ws);
+    auto t = make_tables(p, prec, ws, s);
     g_tab_cache[key] = t;
     return t;
 }
@@ -1430,8 +1401,8 @@ static std::shared_ptr<Tables> cached_tables(int dev, int p, int prec, int ws) {
 // separated by two cells, its own set.
 void build_tables(Mesh &m) {
     upload_constants(m.device);
-    m.tab = cached_tables(m.device, m.opt.p, m.opt.precision, 1);
-    if (m.tc.ws == 2) m.tab2 = cached_tables(m.device, m.opt.p, m.opt.precision, 2);
+    m.tab = cached_tables(m.device, m.opt.p, m.opt.precision, 1, m.stream);
+    if (m.tc.ws == 2) m.tab2 = cached_tables(m.device, m.opt.p, m.opt.precision, 2, m.stream);
     else m.tab2.reset();
 }
 

@@ -389,7 +389,14 @@ void build_p2m_moments(Mesh &m, Tree &t);
 void build_translation_groups(Mesh &m, Tree &t);
 // tensor-core M2L (bem_tc.cu)
 bool tc_m2l_available(const Mesh &m);
-void build_tc_tables(int p, const std::vector<double> &om2l, int nops, std::vector<float> &op);
+// the tensor-core kernel's M2L operators: TC_TABLE_DIM^2 FP32 values per offset
+// class (zero-padded), [in / 4][out][in % 4], so that the kernel writes output
+// coefficient `out` into tensor-memory lane `out` and the 32 lanes of a warp
+// read 4 consecutive input coefficients each from 512 contiguous bytes
+constexpr int TC_TABLE_DIM = 128;
+__host__ __device__ inline int tc_table_index(int in, int out) {
+    return ((in >> 2) * TC_TABLE_DIM + out) * 4 + (in & 3);
+}
 void build_tc_super(Tree &t, const std::vector<int4> &chunks_m2l, cudaStream_t s);
 void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed = false);
 bool use_tc_m2l(const Mesh &m);

@@ -31,7 +31,7 @@
 namespace bem {
 
 constexpr int TC_BN = 128;           // pairs per MMA tile (N)
-constexpr int TC_K = 128;            // padded coefficients (K and M)
+constexpr int TC_K = TC_TABLE_DIM;   // padded coefficients (K and M)
 constexpr int TC_KB = 32;            // K-block: one 128-byte swizzled row of TF32 values
 constexpr int TC_NKB = TC_K / TC_KB; // K-blocks per tile
 constexpr int TC_TMEM_COLS = 512;    // A hi [0,128), A lo [128,256), 2 accumulators of 128
@@ -471,22 +471,6 @@ k_m2l_tc(const float *__restrict__ A_all,
 }
 
 // ---------------------------------------------------------------- host side
-// The M2L operators in FP32, [offset][k / 4][row = output coefficient][k % 4]
-// (k = input coefficient), zero-padded to 128 x 128: the kernel writes row r
-// into tensor-memory lane r (its TF32 hi and lo parts), and the 32 rows of a
-// warp read 4 consecutive coefficients each from 512 contiguous bytes
-void build_tc_tables(int p, const std::vector<double> &om2l, int nops, std::vector<float> &op) {
-    const int nc = (p + 1) * (p + 1);
-    op.assign((size_t)nops * TC_K * TC_K, 0.f);
-    for (int o = 0; o < nops; ++o) {
-        const double *T = &om2l[(size_t)o * nc * nc];
-        float *A = &op[(size_t)o * TC_K * TC_K];
-        for (int row = 0; row < nc; ++row)
-            for (int k = 0; k < nc; ++k)
-                A[((size_t)(k >> 2) * TC_K + row) * 4 + (k & 3)] = (float)T[(size_t)k * nc + row];
-    }
-}
-
 bool tc_m2l_available(const Mesh &m) {
     return m.opt.precision == BEM_MIXED && (m.opt.p + 1) * (m.opt.p + 1) <= TC_K;
 }
