@@ -139,12 +139,12 @@ size_t Mesh::bytes() const {
     b += lamq.bytes() + pan64.bytes() + cn_off.bytes() + cn_col.bytes() + cn_val.bytes() + cnT_off.bytes() + cnT_row.bytes() +
          cnT_val.bytes();
     b += Mtc.bytes() + ctq.bytes() + str32.bytes() + str64.bytes() + near64.bytes() + dpart_f.bytes() +
-         dpart_d.bytes();
+         dpart_d.bytes() + dsrc.bytes();
     b += xs.bytes() + ys.bytes() + zs.bytes() + far_f.bytes() + near_f.bytes() + far_d.bytes() +
          near_d.bytes() + io_a.bytes() + io_b.bytes() + red.bytes();
     b += dev_err.bytes();
     b += V.bytes() + H.bytes() + gv.bytes() + cs.bytes() + sn.bytes() + yv.bytes() + hv.bytes() +
-         part.bytes() + sigma_s.bytes();
+         part.bytes() + sigma_s.bytes() + adj.bytes();
     return b;
 }
 

@@ -11,6 +11,16 @@ template <class T> struct V4T;
 template <> struct V4T<float> { using t = float4; };
 template <> struct V4T<double> { using t = double4; };
 
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// 16-byte copy global -> shared (ok = false writes zero, src-size 0)
+__device__ __forceinline__ void cp_async_16(void *dst, const void *src, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
 // Strength of source i of a pass: the record's weight times the density
 // (A_j w_q dens[panel] for a quadrature point; dens[k], or the charge stored
 // in the record when dens is null, for a charge).

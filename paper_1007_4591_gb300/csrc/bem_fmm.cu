@@ -418,16 +418,6 @@ __global__ void k_apply_far_near(const double *x, const T *far, const double *ne
     y[i] = x[i] + ehat * (v * (1.0 / FOUR_PI));
 }
 
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// 16-byte copy global -> shared (ok = false writes zero, src-size 0)
-__device__ __forceinline__ void cp_async_16(void *dst, const void *src, bool ok) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-
 // Two lanes of T: packed FP32 instructions on sm_100+ (per component the
 // same rounding as the scalar fmaf / fadd / fmul), plain pairs for FP64.
 template <class T> struct Pk;

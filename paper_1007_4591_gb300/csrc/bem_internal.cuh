@@ -323,6 +323,7 @@ struct Mesh {
     DArray<float> Mtc;                 // multipoles split hi|lo for the tensor-core M2L
     DArray<float> dpart_f;             // direct-sum partials (mixed)
     DArray<double> dpart_d;            // direct-sum partials (fp64)
+    DArray<float4> dsrc;               // direct-sum source records of one segment (mixed)
     double *h_pinned = nullptr;        // small pinned host buffer
 
     // GMRES workspace
@@ -330,6 +331,7 @@ struct Mesh {
     // last solve (for the adjoint)
     DArray<double> sigma_s;
     bool have_sigma = false;
+    DArray<double> adj;                // the adjoint gradients' vectors
 
     DArray<int> dev_err;               // device error word (bounded waits that ran out)
     Timers tm;
@@ -427,6 +429,26 @@ void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *ou
 bool charge_direct(const Mesh &m);
 void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out);
 void build_ctq(Mesh &m);
+// All-pairs sums in FP32 with split coordinates (bem_direct.cu), shared by the
+// charge passes and the adjoint: sources and outputs of one call
+enum DirectOut { DO_DN, DO_PHI, DO_PHI_GRAD };  // normal field, potential, potential and gradient
+struct DirectSum {
+    bool dipole = false;           // moments dens[k] nrm[k] instead of strengths
+    bool skip_coincident = false;  // a pair at distance 0 adds nothing
+    DirectOut kind = DO_PHI;
+    int64_t nsrc = 0, ntgt = 0;
+    const double *spos = nullptr, *sw = nullptr, *snrm = nullptr, *dens = nullptr;
+    const int *qpanel = nullptr;   // strengths sw[k] dens[qpanel[k]] (else dens[k], or sw[k] without dens)
+    const double *tpos = nullptr, *tnrm = nullptr;
+};
+// part[split][target] (x 4 with the gradient), split s over the sources [s chunk, (s + 1) chunk)
+void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, float *part);
+// out[n][no] = 1/(4 pi) x the sum over the splits of part[split][n][no], each
+// `group` consecutive splits added in T first
+template <class T>
+void direct_reduce(const T *part, int nsplit, int group, int64_t n, int no, double *out, cudaStream_t s);
+// per panel, the weighted sum of its quadrature points' values
+void panel_wsum(Mesh &m, const double *v, double *out);
 double energy_from_ctq(Mesh &m, const double *sig_s);
 
 // solver pieces (bem_solver.cu)
