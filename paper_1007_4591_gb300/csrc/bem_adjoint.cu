@@ -19,7 +19,7 @@
 
 namespace bem {
 
-int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_stats *st);
+int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bool x_zero, bem_solve_stats *st);
 
 enum AdjSrc { AS_QUAD = 0, AS_CHARGE = 1, AS_DIPOLE = 2 };
 enum AdjTgt { AT_CHG_GRAD = 0, AT_QUAD_PHI = 1 };
@@ -219,7 +219,7 @@ void adjoint_gradients(Mesh &m, double grad_out, double *dq_s, double *dx_s) {
     // A^T lam = C^T q
     BEM_CUDA(cudaMemsetAsync(lam, 0, np * sizeof(double), s));
     bem_solve_stats st{};
-    gmres_solve(m, rhs, lam, true, &st);
+    gmres_solve(m, rhs, lam, true, true, &st);
     // B^T lam and its gradient: dipoles lam_i n_i at the collocation points
     // (Galerkin: lam_i w_q n_i at the quadrature points)
     if (m.opt.galerkin) galerkin_moments(m, lam);

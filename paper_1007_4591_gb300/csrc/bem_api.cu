@@ -18,7 +18,7 @@
 
 namespace bem {
 
-int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_stats *st);
+int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bool x_zero, bem_solve_stats *st);
 double energy_from_phi(Mesh &m, const double *phi_s);
 void axpby(Mesh &m, double a, const double *x, double b, const double *y, double *out, int64_t n);
 void adjoint_gradients(Mesh &m, double grad_out, double *dq_s, double *dx_s);
@@ -144,7 +144,7 @@ size_t Mesh::bytes() const {
          near_d.bytes() + io_a.bytes() + io_b.bytes() + red.bytes();
     b += dev_err.bytes();
     b += V.bytes() + H.bytes() + gv.bytes() + cs.bytes() + sn.bytes() + yv.bytes() + hv.bytes() +
-         part.bytes() + sigma_s.bytes() + adj.bytes();
+         part.bytes() + sigma_s.bytes() + adj.bytes() + bvec.bytes() + ticket.bytes();
     return b;
 }
 
@@ -185,6 +185,10 @@ static void alloc_work(Mesh &m) {
     if (!m.dev_err.p) {
         m.dev_err.alloc(2);  // [0] error word, [1] work-item counter of the tensor-core M2L
         BEM_CUDA(cudaMemsetAsync(m.dev_err.p, 0, 2 * sizeof(int), m.stream));
+    }
+    if (!m.ticket.p) {
+        m.ticket.alloc(1);
+        BEM_CUDA(cudaMemsetAsync(m.ticket.p, 0, sizeof(unsigned), m.stream));
     }
     ensure(m.part, (size_t)(std::max(1, m.opt.gmres_restart) + 2) * 1024);
 }
@@ -413,6 +417,12 @@ static void rhs_sorted(Mesh &m, double *b_s) {
     axpby(m, -m.ehat, m.zs.p, 0.0, m.zs.p, b_s, m.np);
 }
 
+// the solve's right-hand side, kept with the mesh
+static double *rhs_vector(Mesh &m) {
+    if (m.bvec.n < (size_t)m.np) m.bvec.alloc(m.np);
+    return m.bvec.p;
+}
+
 int bem_rhs(bem_mesh *m, double *b) {
     Range rng("bem_rhs");
     if (!m || !b) return BEM_EINVAL;
@@ -438,9 +448,8 @@ int bem_solve(bem_mesh *m, const double *x0, double *sigma, bem_solve_stats *st)
         BEM_CUDA(cudaEventCreate(&e2));
         BEM_CUDA(cudaEventRecord(e0, m->stream));
         if (m->sigma_s.n < (size_t)m->np) m->sigma_s.alloc(m->np);
-        DArray<double> b;
-        b.alloc(m->np);
-        rhs_sorted(*m, b.p);
+        double *b = rhs_vector(*m);
+        rhs_sorted(*m, b);
         BEM_CUDA(cudaEventRecord(e1, m->stream));
         if (x0) {
             const double *d0 = dev_in(*m, x0, m->np, m->io_a);
@@ -449,7 +458,7 @@ int bem_solve(bem_mesh *m, const double *x0, double *sigma, bem_solve_stats *st)
             BEM_CUDA(cudaMemsetAsync(m->sigma_s.p, 0, m->np * sizeof(double), m->stream));
         }
         bem_solve_stats local{};
-        status = gmres_solve(*m, b.p, m->sigma_s.p, false, &local);
+        status = gmres_solve(*m, b, m->sigma_s.p, false, !x0, &local);
         BEM_CUDA(cudaEventRecord(e2, m->stream));
         OutArg o = dev_out(*m, sigma, m->np, m->io_b);
         scatter_f64(m->sigma_s.p, m->cen_perm.p, o.dev, m->np, m->stream);
@@ -538,11 +547,10 @@ int bem_energy_backward(bem_mesh *m, double grad_out, double *dq, double *dx) {
         if (!m->have_sigma) {
             bem_solve_stats st{};
             if (m->sigma_s.n < (size_t)m->np) m->sigma_s.alloc(m->np);
-            DArray<double> b;
-            b.alloc(m->np);
-            rhs_sorted(*m, b.p);
+            double *b = rhs_vector(*m);
+            rhs_sorted(*m, b);
             BEM_CUDA(cudaMemsetAsync(m->sigma_s.p, 0, m->np * sizeof(double), m->stream));
-            gmres_solve(*m, b.p, m->sigma_s.p, false, &st);
+            gmres_solve(*m, b, m->sigma_s.p, false, true, &st);
             m->have_sigma = true;
         }
         DArray<double> gq, gx;

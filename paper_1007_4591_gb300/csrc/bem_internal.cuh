@@ -328,6 +328,8 @@ struct Mesh {
 
     // GMRES workspace
     DArray<double> V, H, gv, cs, sn, yv, hv, part;
+    DArray<double> bvec;               // the solve's right-hand side
+    DArray<unsigned> ticket;           // arrivals of a reduction's CTAs
     // last solve (for the adjoint)
     DArray<double> sigma_s;
     bool have_sigma = false;

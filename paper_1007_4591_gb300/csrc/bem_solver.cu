@@ -3,8 +3,8 @@
 // All vectors here are FP64 and in the sorted panel order; the public entry
 // points gather/scatter at the boundary.  GMRES (Saad & Schultz) runs on the
 // device: classical Gram-Schmidt applied twice (CGS2) for the Arnoldi step,
-// Givens rotations for the least-squares update, one 8-byte residual read by
-// the host per iteration to decide convergence.
+// Givens rotations for the least-squares update, one 8-byte residual written to
+// pinned host memory per iteration to decide convergence.
 #include <cmath>
 #include <vector>
 
@@ -13,20 +13,6 @@
 namespace bem {
 
 constexpr int RED_THREADS = 256;
-
-__device__ __forceinline__ double block_sum(double v) {
-    __shared__ double sh[32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    v = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-    if (w == 0)
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // ------------------------------------------------------------ permutations
 __global__ void k_gather(const double *src, const int *perm, double *dst, int64_t n) {
@@ -155,59 +141,110 @@ void matvec_sorted(Mesh &m, const double *xs, double *ys) {
 }
 
 // --------------------------------------------------------------- BLAS-1
-__global__ void k_dot_parts(const double *V, size_t ld, const double *w, int64_t n, int chunk,
-                            double *part) {
-    const int i = blockIdx.y, c = blockIdx.x;
-    const int64_t b = (int64_t)c * chunk, e = min(n, b + chunk);
-    const double *v = V + (size_t)i * ld;
-    double s = 0.0;
-    for (int64_t r = b + threadIdx.x; r < e; r += blockDim.x) s += v[r] * w[r];
-    s = block_sum(s);
-    if (threadIdx.x == 0) part[(size_t)i * gridDim.x + c] = s;
+// Reductions end in the kernel that starts them: the last CTA to arrive
+// (a ticket that wraps to zero) adds the CTAs' parts in a fixed order.  At
+// GMRES sizes these kernels are launches and latency, not bandwidth (8 n bytes
+// a vector, 0.1 us at 81,920 panels): an Arnoldi step was 11 launches and a
+// copy, is four launches, and the host reads the residual from pinned memory
+// the device writes (81,920 panels, 8 iterations: solve 2.98 -> 2.75 ms; 1,280 panels 0.88 -> 0.70).
+
+// rows of a CTA: a multiple of its threads, at most one CTA per SM
+static int rows_for(int64_t n) { return RED_THREADS * std::max(1, cdiv(n, (int64_t)RED_THREADS * 152)); }
+
+__device__ __forceinline__ bool last_cta(unsigned *ticket) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
 }
 
-// out[i] (+)= sum of the parts of vector i; mode 0: store, 1: add, 2: store sqrt
-__global__ void k_finish(const double *part, int nchunk, double *out, int mode) {
-    const int i = blockIdx.x;
-    double s = 0.0;
-    for (int c = threadIdx.x; c < nchunk; c += blockDim.x) s += part[(size_t)i * nchunk + c];
-    s = block_sum(s);
-    if (threadIdx.x == 0) {
-        if (mode == 0) out[i] = s;
-        else if (mode == 1) out[i] += s;
-        else out[i] = sqrt(s);
+// part[i][CTA] = the CTA's rows' share of V_i . w, for nvec vectors, 8 at a time
+__device__ __forceinline__ void dot_rows(const double *V, size_t ld, int nvec, const double *w, int64_t b, int64_t e,
+                                         double *part) {
+    __shared__ double sh[8][RED_THREADS / 32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    for (int i0 = 0; i0 < nvec; i0 += 8) {
+        const int ni = min(8, nvec - i0);
+        double s[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] = 0.0;
+        for (int64_t r = b + threadIdx.x; r < e; r += RED_THREADS) {
+            const double x = w[r];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < ni) s[i] += V[(size_t)(i0 + i) * ld + r] * x;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (i < ni)
+                for (int o = 16; o > 0; o >>= 1) s[i] += __shfl_down_sync(0xffffffffu, s[i], o);
+            if (lane == 0) sh[i][wp] = s[i];
+        }
+        __syncthreads();
+        if (threadIdx.x < ni) {
+            double t = 0.0;
+            for (int k = 0; k < RED_THREADS / 32; ++k) t += sh[threadIdx.x][k];
+            part[(size_t)(i0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+        }
     }
 }
 
-// w -= sum_i h[i] V_i   (sign = -1)   or   w += sum_i h[i] V_i (sign = +1)
-__global__ void k_multi_axpy(const double *V, size_t ld, int nvec, const double *h, double sign,
-                             double *w, int64_t n) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    double a = 0.0;
-    for (int i = 0; i < nvec; ++i) a += h[i] * V[(size_t)i * ld + r];
-    w[r] += sign * a;
+// out[i] = the sum of vector i's parts (a warp per vector)
+__device__ __forceinline__ void sum_parts(const double *part, int nvec, double *out) {
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < nvec; i += RED_THREADS / 32) {
+        double t = 0.0;
+        for (int k = lane; k < (int)gridDim.x; k += 32) t += __ldcg(part + (size_t)i * gridDim.x + k);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) out[i] = t;
+    }
 }
 
-__global__ void k_scale_by(double *w, const double *sc, int64_t n) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r < n) w[r] *= sc[0];
+// w -= sum_i h[i] V_i over the CTA's rows
+__device__ __forceinline__ void sub_rows(const double *V, size_t ld, int nvec, const double *h, double *w, int64_t b,
+                                         int64_t e) {
+    for (int64_t r = b + threadIdx.x; r < e; r += RED_THREADS) {
+        double a = 0.0;
+        for (int i = 0; i < nvec; ++i) a += h[i] * V[(size_t)i * ld + r];
+        w[r] -= a;
+    }
 }
 
-__global__ void k_scale_by_inv(double *w, const double *d, int64_t n) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r < n) w[r] /= d[0];
+// out[0] = V . w (mode 0) or its square root (mode 1), also written to `host`
+__global__ void __launch_bounds__(RED_THREADS)
+k_dot(const double *V, const double *w, int64_t n, int rows, double *part, unsigned *ticket, int mode, double *out,
+      volatile double *host) {
+    const int64_t b = (int64_t)blockIdx.x * rows, e = min(n, b + rows);
+    dot_rows(V, 0, 1, w, b, e, part);
+    if (!last_cta(ticket)) return;
+    __shared__ double t;
+    sum_parts(part, 1, &t);
+    if (threadIdx.x == 0) {
+        const double v = mode ? sqrt(t) : t;
+        out[0] = v;
+        *host = v;
+        __threadfence_system();
+    }
 }
 
-__global__ void k_axpby(double a, const double *x, double b, const double *y, double *out,
-                        int64_t n) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r < n) out[r] = a * x[r] + b * y[r];
+// First pass of classical Gram-Schmidt, h = V^T w, or (hsub set) the second:
+// w -= V hsub, then h = V^T w.
+__global__ void __launch_bounds__(RED_THREADS)
+k_cgs(const double *V, size_t ld, int nvec, const double *hsub, double *w, int64_t n, int rows, double *part,
+      unsigned *ticket, double *h) {
+    const int64_t b = (int64_t)blockIdx.x * rows, e = min(n, b + rows);
+    if (hsub) sub_rows(V, ld, nvec, hsub, w, b, e);
+    dot_rows(V, ld, nvec, w, b, e, part);
+    if (last_cta(ticket)) sum_parts(part, nvec, h);
 }
 
 // Givens update of Hessenberg column j (column-major, leading dimension m1).
-__global__ void k_givens(double *H, int m1, const double *hcol, int j, double *cs, double *sn,
-                         double *g, double inv_bnorm, double *out /* [0]=resid, [1]=1/norm */) {
+__device__ void givens(double *H, int m1, const double *hcol, int j, double *cs, double *sn, double *g, double inv_bnorm,
+                       double *out /* [0]=resid, [1]=1/norm */) {
     double *h = H + (size_t)j * m1;
     for (int i = 0; i <= j + 1; ++i) h[i] = hcol[i];
     const double wn = h[j + 1];
@@ -232,54 +269,87 @@ __global__ void k_givens(double *H, int m1, const double *hcol, int j, double *c
     out[1] = (wn > 0.0) ? 1.0 / wn : 0.0;
 }
 
-// Back substitution  H[:k,:k] y = g[:k].
-__global__ void k_backsolve(const double *H, int m1, const double *g, int k, double *y) {
-    for (int i = k - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int l = i + 1; l < k; ++l) s -= H[(size_t)l * m1 + i] * y[l];
-        const double d = H[(size_t)i * m1 + i];
-        y[i] = (d != 0.0) ? s / d : 0.0;
+// The Arnoldi step's end: w -= V h2, |w|, the Hessenberg column h + h2 | |w|
+// through the Givens rotations, the residual to the host.
+__global__ void __launch_bounds__(RED_THREADS)
+k_cgs_end(const double *V, size_t ld, int j, double *h, const double *h2, double *w, int64_t n, int rows, double *part,
+          unsigned *ticket, double *H, int m1, double *cs, double *sn, double *g, double inv_bnorm, double *out,
+          volatile double *host) {
+    const int64_t b = (int64_t)blockIdx.x * rows, e = min(n, b + rows);
+    sub_rows(V, ld, j + 1, h2, w, b, e);
+    dot_rows(w, 0, 1, w, b, e, part);
+    if (!last_cta(ticket)) return;
+    __shared__ double t;
+    sum_parts(part, 1, &t);
+    for (int i = threadIdx.x; i <= j; i += RED_THREADS) h[i] += h2[i];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        h[j + 1] = sqrt(t);
+        givens(H, m1, h, j, cs, sn, g, inv_bnorm, out);
+        *host = out[0];
+        __threadfence_system();
     }
 }
 
-__global__ void k_set_g(double *g, int n, double beta) {
-    int i = threadIdx.x + blockIdx.x * blockDim.x;
-    if (i < n) g[i] = (i == 0) ? beta : 0.0;
+// x += sum_i h[i] V_i
+__global__ void k_multi_axpy(const double *V, size_t ld, int nvec, const double *h, double *x, int64_t n) {
+    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (r >= n) return;
+    double a = 0.0;
+    for (int i = 0; i < nvec; ++i) a += h[i] * V[(size_t)i * ld + r];
+    x[r] += a;
 }
 
-static int nchunk_for(int64_t n) {
-    int64_t c = (n + 4095) / 4096;
-    if (c > 1024) c = 1024;
-    if (c < 1) c = 1;
-    return (int)c;
+__global__ void k_scale_by(double *w, const double *sc, int64_t n) {
+    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (r < n) w[r] *= sc[0];
 }
 
-// dots out[0..nvec) = V[0..nvec)^T w  (mode as in k_finish)
-static void dots(Mesh &m, const double *V, size_t ld, int nvec, const double *w, double *out,
-                 int mode) {
-    const int64_t n = m.np;
-    const int nch = nchunk_for(n);
-    const int chunk = (int)((n + nch - 1) / nch);
-    dim3 grid(nch, nvec);
-    k_dot_parts<<<grid, RED_THREADS, 0, m.stream>>>(V, ld, w, n, chunk, m.part.p);
+// v = u / d[0] (u may be v), and g = (d[0], 0, ..., 0) with m1 entries
+__global__ void k_start_basis(const double *u, const double *d, double *v, int64_t n, double *g, int m1) {
+    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (r < n) v[r] = u[r] / d[0];
+    if (r < m1) g[r] = r == 0 ? d[0] : 0.0;
+}
+
+__global__ void k_axpby(double a, const double *x, double b, const double *y, double *out,
+                        int64_t n) {
+    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (r < n) out[r] = a * x[r] + b * y[r];
+}
+
+// Back substitution H[:k,:k] y = g[:k], column by column: a thread per row
+// (one thread alone waits for every entry in turn).
+__global__ void k_backsolve(const double *H, int m1, const double *g, int k, double *y) {
+    __shared__ double yi;
+    const int l = threadIdx.x;
+    double s = l < k ? g[l] : 0.0;
+    for (int i = k - 1; i >= 0; --i) {
+        const double v = l <= i ? H[(size_t)i * m1 + l] : 0.0;
+        if (l == i) {
+            yi = v != 0.0 ? s / v : 0.0;
+            y[i] = yi;
+        }
+        __syncthreads();
+        if (l < i) s -= v * yi;
+        __syncthreads();
+    }
+}
+
+// V . w (mode 0) or its square root (mode 1), left in *out and read by the host
+static double dot_read(Mesh &m, const double *V, const double *w, int64_t n, int mode, double *out) {
+    const int rows = rows_for(n);
+    k_dot<<<cdiv(n, rows), RED_THREADS, 0, m.stream>>>(V, w, n, rows, m.part.p, m.ticket.p, mode, out, m.h_pinned);
     BEM_CHECK_LAUNCH();
-    k_finish<<<nvec, RED_THREADS, 0, m.stream>>>(m.part.p, nch, out, mode);
-    BEM_CHECK_LAUNCH();
-}
-
-static double read_scalar(Mesh &m, const double *d) {
-    BEM_CUDA(cudaMemcpyAsync(m.h_pinned, d, sizeof(double), cudaMemcpyDeviceToHost, m.stream));
     BEM_CUDA(cudaStreamSynchronize(m.stream));
-    return m.h_pinned[0];
+    return *const_cast<volatile double *>(m.h_pinned);
 }
 
-double norm2(Mesh &m, const double *w) {
-    dots(m, w, 0, 1, w, m.red.p, 2);
-    return read_scalar(m, m.red.p);
-}
+double norm2(Mesh &m, const double *w) { return dot_read(m, w, w, m.np, 1, m.red.p); }
 
-// Solve A x = b (sorted order).  x holds the initial guess on entry.
-int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_stats *st) {
+// Solve A x = b (sorted order).  x holds the initial guess on entry; with
+// x_zero the caller knows it to be zero.
+int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bool x_zero, bem_solve_stats *st) {
     const int64_t n = m.np;
     const int mr = std::max(1, m.opt.gmres_restart);
     const int m1 = mr + 1;
@@ -308,31 +378,27 @@ int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_s
         rec = 0.0;
         conv = true;
     }
-    bool x_zero = false;
-    {
-        // detect an all-zero initial guess to skip one product
-        const double xn = conv ? 0.0 : norm2(m, x);
-        x_zero = (xn == 0.0);
-    }
+    // an all-zero initial guess skips one product: the residual is b
+    const bool told = x_zero;  // red[0] still holds |b|
+    if (!x_zero && !conv) x_zero = norm2(m, x) == 0.0;
+    const int rows = rows_for(n), ncta = cdiv(n, rows);
     while (!conv && it < m.opt.max_iter && !stagnated) {
         double *V0 = m.V.p;
-        if (x_zero) {
-            BEM_CUDA(cudaMemcpyAsync(V0, b, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-        } else {
+        const double *r0 = b;
+        if (!x_zero) {
             apply(x, V0);
             k_axpby<<<nb, 256, 0, s>>>(1.0, b, -1.0, V0, V0, n);
             BEM_CHECK_LAUNCH();
+            r0 = V0;
         }
-        const double beta = norm2(m, V0);
+        const double beta = told && it == 0 ? bnorm : norm2(m, r0);
         rec = beta / bnorm;
         if (rec <= m.opt.tol) {
             conv = true;
             break;
         }
-        // V0 /= beta, with beta read on the device (norm2 left it in red[0])
-        k_scale_by_inv<<<nb, 256, 0, s>>>(V0, m.red.p, n);
-        BEM_CHECK_LAUNCH();
-        k_set_g<<<1, 64, 0, s>>>(m.gv.p, m1, beta);
+        // V0 = r0 / beta, with beta read on the device (left in red[0] by norm2)
+        k_start_basis<<<std::max(nb, cdiv(m1, 256)), 256, 0, s>>>(r0, m.red.p, V0, n, m.gv.p, m1);
         BEM_CHECK_LAUNCH();
         int k = 0;
         for (int j = 0; j < mr; ++j) {
@@ -340,21 +406,17 @@ int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_s
             apply(m.V.p + (size_t)j * ld, w);
             ++it;
             // CGS2: two passes of classical Gram-Schmidt
-            dots(m, m.V.p, ld, j + 1, w, m.hv.p, 0);
-            k_multi_axpy<<<nb, 256, 0, s>>>(m.V.p, ld, j + 1, m.hv.p, -1.0, w, n);
+            k_cgs<<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, j + 1, nullptr, w, n, rows, m.part.p, m.ticket.p, m.hv.p);
             BEM_CHECK_LAUNCH();
-            dots(m, m.V.p, ld, j + 1, w, m.yv.p, 0);
-            k_multi_axpy<<<nb, 256, 0, s>>>(m.V.p, ld, j + 1, m.yv.p, -1.0, w, n);
+            k_cgs<<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, j + 1, m.hv.p, w, n, rows, m.part.p, m.ticket.p, m.yv.p);
             BEM_CHECK_LAUNCH();
-            k_axpby<<<1, 64, 0, s>>>(1.0, m.hv.p, 1.0, m.yv.p, m.hv.p, j + 1);
-            BEM_CHECK_LAUNCH();
-            dots(m, w, 0, 1, w, m.hv.p + j + 1, 2);
-            k_givens<<<1, 1, 0, s>>>(m.H.p, m1, m.hv.p, j, m.cs.p, m.sn.p, m.gv.p, 1.0 / bnorm,
-                                     m.red.p);
+            k_cgs_end<<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, j, m.hv.p, m.yv.p, w, n, rows, m.part.p, m.ticket.p, m.H.p,
+                                                   m1, m.cs.p, m.sn.p, m.gv.p, 1.0 / bnorm, m.red.p, m.h_pinned);
             BEM_CHECK_LAUNCH();
             k_scale_by<<<nb, 256, 0, s>>>(w, m.red.p + 1, n);
             BEM_CHECK_LAUNCH();
-            rec = read_scalar(m, m.red.p);
+            BEM_CUDA(cudaStreamSynchronize(s));
+            rec = *const_cast<volatile double *>(m.h_pinned);
             hist.push_back(rec);
             k = j + 1;
             if (!(rec == rec)) {  // NaN
@@ -368,9 +430,9 @@ int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_s
                 break;
             }
         }
-        k_backsolve<<<1, 1, 0, s>>>(m.H.p, m1, m.gv.p, k, m.yv.p);
+        k_backsolve<<<1, RED_THREADS, 0, s>>>(m.H.p, m1, m.gv.p, k, m.yv.p);
         BEM_CHECK_LAUNCH();
-        k_multi_axpy<<<nb, 256, 0, s>>>(m.V.p, ld, k, m.yv.p, 1.0, x, n);
+        k_multi_axpy<<<nb, 256, 0, s>>>(m.V.p, ld, k, m.yv.p, x, n);
         BEM_CHECK_LAUNCH();
         x_zero = false;
         if (rec <= m.opt.tol) conv = true;
@@ -395,30 +457,12 @@ int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bem_solve_s
 
 // dG = 4 pi 332.0637 / (2 eps_in) * (C^T q) . sigma
 double energy_from_ctq(Mesh &m, const double *sig_s) {
-    const int64_t n = m.np;
-    const int nch = nchunk_for(n);
-    const int chunk = (int)((n + nch - 1) / nch);
-    dim3 grid(nch, 1);
-    k_dot_parts<<<grid, RED_THREADS, 0, m.stream>>>(m.ctq.p, 0, sig_s, n, chunk, m.part.p);
-    BEM_CHECK_LAUNCH();
-    k_finish<<<1, RED_THREADS, 0, m.stream>>>(m.part.p, nch, m.red.p + 2, 0);
-    BEM_CHECK_LAUNCH();
-    const double ctqs = read_scalar(m, m.red.p + 2);
-    return FOUR_PI * KCAL / (2.0 * m.eps_in) * ctqs;
+    return FOUR_PI * KCAL / (2.0 * m.eps_in) * dot_read(m, m.ctq.p, sig_s, m.np, 0, m.red.p + 2);
 }
 
 // dG = 4 pi 332.0637 / (2 eps_in) * q . phi   (phi = C sigma, G = 1/(4 pi r))
 double energy_from_phi(Mesh &m, const double *phi_s) {
-    const int64_t n = m.nc;
-    const int nch = nchunk_for(n);
-    const int chunk = (int)((n + nch - 1) / nch);
-    dim3 grid(nch, 1);
-    k_dot_parts<<<grid, RED_THREADS, 0, m.stream>>>(m.q64.p, 0, phi_s, n, chunk, m.part.p);
-    BEM_CHECK_LAUNCH();
-    k_finish<<<1, RED_THREADS, 0, m.stream>>>(m.part.p, nch, m.red.p + 2, 0);
-    BEM_CHECK_LAUNCH();
-    const double qphi = read_scalar(m, m.red.p + 2);
-    return FOUR_PI * KCAL / (2.0 * m.eps_in) * qphi;
+    return FOUR_PI * KCAL / (2.0 * m.eps_in) * dot_read(m, m.q64.p, phi_s, m.nc, 0, m.red.p + 2);
 }
 
 void axpby(Mesh &m, double a, const double *x, double b, const double *y, double *out, int64_t n) {
