@@ -200,15 +200,19 @@ __global__ void k_gradients(const double *cs4, const double *bl4, const double *
 
 void build_qp_of_panel(Mesh &m);
 
+AdjointVectors adjoint_vectors(Mesh &m) {
+    const size_t nc = (size_t)m.nc, np = (size_t)m.np, need = 12 * nc + 2 * np + (size_t)m.nqp;
+    if (m.adj.n < need) m.adj.alloc(need);
+    double *p = m.adj.p;
+    return AdjointVectors{p, p + 4 * nc, p + 8 * nc, p + 9 * nc, p + 12 * nc, p + 12 * nc + np, p + 12 * nc + 2 * np};
+}
+
 void adjoint_gradients(Mesh &m, double grad_out, double *dq_s, double *dx_s) {
     cudaStream_t s = m.stream;
     build_qp_of_panel(m);
     const int64_t np = m.np, nc = m.nc;
-    // kept between calls: (phi, grad) of C sigma and of B^T lam, lam, C^T q
-    // and the charges' potential at the quadrature points
-    const size_t need = (size_t)nc * 8 + (size_t)np * 2 + (size_t)m.nqp;
-    if (m.adj.n < need) m.adj.alloc(need);
-    double *cs4 = m.adj.p, *bl4 = cs4 + 4 * nc, *lam = bl4 + 4 * nc, *rhs = lam + np, *psi = rhs + np;
+    const AdjointVectors v = adjoint_vectors(m);
+    double *cs4 = v.cs4, *bl4 = v.bl4, *lam = v.lam, *rhs = v.rhs, *psi = v.psi;
     // C sigma and its gradient at the charges
     direct_adjoint(m, AS_QUAD, AT_CHG_GRAD, m.sigma_s.p, cs4);
     charge_near_phi(m, m.sigma_s.p, cs4, 4, 4);

@@ -296,7 +296,7 @@ int bem_mesh_create(const double *panels, int64_t n_p, const double *charges, in
         st.mark("translation tables");
         build_translation_groups(*m, m->tp);
         st.mark("panel tree: translation groups, near-field order");
-        build_translation_groups(*m, m->tc);
+        if (m->tc.nleaf > 0) build_translation_groups(*m, m->tc);
         st.mark("charge tree: translation groups, near-field order");
         alloc_work(*m);
         st.mark("work buffers");
@@ -369,7 +369,7 @@ int bem_set_charges(bem_mesh *m, const double *charges, int64_t n_c) {
         }
         rebuild_charge_tree(*m, dc);
         build_tables(*m);  // the charge tree's separation may have changed
-        build_translation_groups(*m, m->tc);
+        if (m->tc.nleaf > 0) build_translation_groups(*m, m->tc);
         alloc_work(*m);
         build_charge_near(*m);
         build_ctq(*m);
@@ -553,18 +553,16 @@ int bem_energy_backward(bem_mesh *m, double grad_out, double *dq, double *dx) {
             gmres_solve(*m, b, m->sigma_s.p, false, true, &st);
             m->have_sigma = true;
         }
-        DArray<double> gq, gx;
-        gq.alloc(m->nc);
-        gx.alloc((size_t)m->nc * 3);
-        adjoint_gradients(*m, grad_out, gq.p, gx.p);
+        const AdjointVectors v = adjoint_vectors(*m);
+        adjoint_gradients(*m, grad_out, v.gq, v.gx);
         if (dq) {
             OutArg o = dev_out(*m, dq, m->nc, m->io_a);
-            scatter_f64(gq.p, m->chg_perm.p, o.dev, m->nc, m->stream);
+            scatter_f64(v.gq, m->chg_perm.p, o.dev, m->nc, m->stream);
             finish_out(*m, o);
         }
         if (dx) {
             OutArg o = dev_out(*m, dx, (size_t)m->nc * 3, m->io_b);
-            scatter_rows3(gx.p, m->chg_perm.p, o.dev, m->nc, m->stream);
+            scatter_rows3(v.gx, m->chg_perm.p, o.dev, m->nc, m->stream);
             finish_out(*m, o);
         }
         sync(*m);

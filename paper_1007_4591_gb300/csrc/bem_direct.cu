@@ -459,10 +459,9 @@ void build_ctq(Mesh &m) {
     m.ctq_ok = false;
     if (m.nc == 0 || !charge_direct(m)) return;
     if (m.ctq.n < (size_t)m.np) m.ctq.alloc(m.np);
-    DArray<double> psi;
-    psi.alloc(m.nqp);
-    direct_pass(m, SRC_CHARGE, TGT_QUAD_PHI, nullptr, psi.p);
-    panel_wsum(m, psi.p, m.ctq.p);
+    double *psi = adjoint_vectors(m).psi;
+    direct_pass(m, SRC_CHARGE, TGT_QUAD_PHI, nullptr, psi);
+    panel_wsum(m, psi, m.ctq.p);
     charge_near_ct(m, m.q64.p, m.ctq.p);
     BEM_CUDA(cudaStreamSynchronize(m.stream));
     m.ctq_ok = true;

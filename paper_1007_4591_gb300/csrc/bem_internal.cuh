@@ -431,6 +431,12 @@ void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *ou
 bool charge_direct(const Mesh &m);
 void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out);
 void build_ctq(Mesh &m);
+// the adjoint gradients' vectors, kept with the mesh: (phi, grad) of C sigma and
+// of B^T lam, the gradients, lam, C^T q, the charges' potential at the points
+struct AdjointVectors {
+    double *cs4, *bl4, *gq, *gx, *lam, *rhs, *psi;
+};
+AdjointVectors adjoint_vectors(Mesh &m);
 // All-pairs sums in FP32 with split coordinates (bem_direct.cu), shared by the
 // charge passes and the adjoint: sources and outputs of one call
 enum DirectOut { DO_DN, DO_PHI, DO_PHI_GRAD };  // normal field, potential, potential and gradient

@@ -732,6 +732,11 @@ static void build_charges(Mesh &m, const double *d_charges) {
         BEM_CUDA(cudaStreamSynchronize(s));
     }
     m.tc = Tree();
+    // Direct charge sums take no tree, and the exact charge-panel pairs find
+    // theirs through it: without those nothing reads it (81,920 panels, 2,000
+    // charges: bem_set_charges 5.1 -> 0.83 ms).  Sets so large that
+    // the near field's work list could refuse them still go through it.
+    if (charge_direct(m) && !charge_near_on(m) && m.nc + m.nqp < (1 << 23)) return;
     SetKeys cen{m.cen_key.p, m.np}, qp{m.qp_key.p, m.nqp}, ch{m.chg_key.p, m.nc};
     // Point charges sit anywhere in their cells (on a corner, as the Born
     // ion's does), where a one-cell separation converges only like

@@ -65,3 +65,25 @@ def test_sources_in_several_segments(pkg):
     with pkg.Mesh(m.panels, m.charges, m.eps_in, m.eps_out) as g:
         _, phi = g.energy(torch.from_numpy(sig).cuda(), want_phi=True)
         close(phi.cpu().numpy(), P.c(sig) / m.eps_in, 2e-6, what="C s")
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_charge_sets_replaced_without_a_charge_tree(pkg, fp64):
+    """Direct charge sums keep no charge tree: sets of other sizes (none, more,
+    fewer) give what a mesh made with them gives."""
+    m = _mol(2, 40)
+    tol = 1e-12 if fp64 else 2e-6
+    with pkg.Mesh(m.panels, m.charges, m.eps_in, m.eps_out, precision=int(fp64), depth=2) as g:
+        sig = torch.from_numpy(np.random.default_rng(3).standard_normal(m.n_p)).cuda()
+        g.set_charges(np.zeros((0, 4)))
+        assert float(g.rhs().abs().max()) == 0.0 and g.energy(sig) == 0.0
+        for n_c in (600, 3):
+            w = _mol(2, n_c)
+            P = oracle.Problem(w.panels, w.charges, w.eps_in, w.eps_out)
+            g.set_charges(w.charges)
+            close(g.rhs().cpu().numpy(), -P.ehat * P.bq(), tol, what="B q")
+            close(g.energy(sig, want_phi=True)[1].cpu().numpy(), P.c(sig.cpu().numpy()) / w.eps_in, tol, what="C s")
+            dq, dx = g.energy_backward()
+            _, rq, rx = P.gradients()[:3]
+            close(dq.cpu().numpy(), rq, 1e-5, what="dq")  # p = 10 products
+            close(dx.cpu().numpy(), rx, 1e-5, what="dx")
