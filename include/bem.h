@@ -298,9 +298,9 @@ int bem_set_profiling(bem_mesh *mesh, int enable);
 int bem_last_phase_ms(const bem_mesh *mesh, double *times);
 
 /* Inside the M2L phase of the last profiled bem_matvec with the tensor-core
- * M2L: device time (ms) of the multipole split (k_split_m), of the
- * tensor-core kernel (k_m2l_tc, which adds the rows into their targets) and
- * a third entry kept at 0 (there is no separate summation kernel).
+ * M2L: a first entry near 0 (the kernel splits the multipoles itself), the
+ * device time (ms) of the tensor-core kernel (k_m2l_tc, which adds the rows
+ * into their targets) and a third entry kept at 0.
  * times[3]; zeros if the product had no tensor-core M2L.  BEM_EINVAL if
  * profiling is off. */
 int bem_last_m2l_ms(const bem_mesh *mesh, double *times);

@@ -138,7 +138,7 @@ size_t Mesh::bytes() const {
     b += Mf.bytes() + Lf.bytes() + Md.bytes() + Ld.bytes();
     b += lamq.bytes() + pan64.bytes() + cn_off.bytes() + cn_col.bytes() + cn_val.bytes() + cnT_off.bytes() + cnT_row.bytes() +
          cnT_val.bytes();
-    b += Mtc.bytes() + ctq.bytes() + str32.bytes() + str64.bytes() + near64.bytes() + dpart_f.bytes() +
+    b += ctq.bytes() + str32.bytes() + str64.bytes() + near64.bytes() + dpart_f.bytes() +
          dpart_d.bytes() + dsrc.bytes();
     b += xs.bytes() + ys.bytes() + zs.bytes() + far_f.bytes() + near_f.bytes() + far_d.bytes() +
          near_d.bytes() + io_a.bytes() + io_b.bytes() + red.bytes();
@@ -168,9 +168,6 @@ static void alloc_work(Mesh &m) {
         ensure(m.Ld, ncell * nc);
         ensure(m.far_d, nt);
         ensure(m.near_d, nt);
-    }
-    if (tc_m2l_available(m)) {
-        ensure(m.Mtc, tc_staging_floats(m));
     }
     // near-field source pairs: each leaf padded to an even count
     const size_t nsrc = (size_t)std::max<int64_t>(m.nqp, m.nc) + (size_t)std::max(m.tp.nleaf, m.tc.nleaf) + 4;

@@ -1408,7 +1408,7 @@ const Tables &tables_for(const Mesh &m, const Tree &t) {
 // shared memory, 8 x 4 outputs per thread, then scattered with coalesced
 // atomic adds (a warp adds 32 consecutive coefficients of one cell).
 constexpr int TR_BM = 128, TR_THREADS = 256;
-constexpr int TR_THREADS_TREE = 256;  // M2M / L2L kernels (chunks of TR_BN_TREE pairs)
+constexpr int TR_THREADS_TREE = 128;  // M2M / L2L kernels (chunks of TR_BN_TREE pairs)
 constexpr int TR_BN_M2L = 64;  // pairs per chunk for M2L (many pairs per offset class)
 constexpr int TR_BN_TREE = 32; // pairs per chunk for M2M / L2L (8 operators per level)
 template <class T> struct TrBK;
@@ -1537,28 +1537,28 @@ k_translate(const T *__restrict__ ops, int nc, int cs, const int4 *__restrict__ 
 
 // M2M / L2L: out[p_out[j]] += Op[octant] . in[p_in[j]] for a chunk of up to
 // BN pairs of one operator.  The level's few thousand translations are
-// latency-bound, so the CTA copies the whole operator block (nc x TR_BM) and
+// latency-bound, so the CTA copies the whole operator block (nc x BM) and
 // the chunk's BN input rows to shared memory in one round of 16-byte
-// cp.async, then each thread forms 8 rows x (BN / 16) pair columns (columns
-// strided by 16; input rows padded to 4 mod 32 words: at most 2-way bank
+// cp.async, then each thread forms RPT rows x BN / NTX pair columns (columns
+// strided by NTX; input rows padded to 4 mod 32 words: at most 2-way bank
 // conflicts) and the results leave as coalesced atomic adds.
-template <class T, int BN, int NTH, int BM>
+template <class T, int BN, int NTH, int BM, int RPT>
 __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, int nc, int cs, int ldb, int4 ch,
                                                      int rb, const int *__restrict__ p_out,
                                                      const int *__restrict__ p_in, const T *__restrict__ in,
                                                      T *__restrict__ out, unsigned char *smraw, int *s_in,
                                                      int *s_out) {
-    constexpr int TR_BM = BM;       // output rows of this CTA
-    constexpr int NTY = TR_BM / 8;  // row groups of 8
-    constexpr int NTX = NTH / NTY;  // column groups
-    constexpr int CPT = BN / NTX;   // columns per thread
+    constexpr int TR_BM = BM;         // output rows of this CTA
+    constexpr int NTY = TR_BM / RPT;  // row groups
+    constexpr int NTX = NTH / NTY;    // column groups
+    constexpr int CPT = BN / NTX;     // columns per thread
     static_assert(NTH % NTY == 0 && BN % NTX == 0, "tree translate tiling");
     constexpr int VEC = 16 / (int)sizeof(T);
     T *As = reinterpret_cast<T *>(smraw);  // [nc][TR_BM]
     T *Bs = As + (size_t)nc * TR_BM;       // [BN][ldb]
     T *Cs = As;                            // [BN][TR_BM + 1] (epilogue)
     const T *Tt = ops + (size_t)ch.x * nc * cs;
-    // a warp covers 8 pair columns x 4 row groups: its input-row loads hit 8
+    // a warp covers 8 pair columns and 4 row groups: its input-row loads hit 8
     // different banks and its operator loads one 128-byte span
     static_assert(NTX % 8 == 0, "tree translate thread map");
     const int tid = threadIdx.x, rest = tid >> 3, ty = rest % NTY, tx = (tid & 7) + 8 * (rest / NTY);
@@ -1588,24 +1588,24 @@ __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, 
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
-    T acc[8][CPT];
+    T acc[RPT][CPT];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < RPT; ++r)
 #pragma unroll
         for (int c = 0; c < CPT; ++c) acc[r][c] = 0;
 #pragma unroll 4
     for (int k = 0; k < nc; ++k) {
-        T a[8], b[CPT];
+        T a[RPT], b[CPT];
 #pragma unroll
-        for (int q = 0; q < 8; q += VEC) {
+        for (int q = 0; q < RPT; q += VEC) {
             if constexpr (sizeof(T) == 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(As + (size_t)k * TR_BM + ty * 8 + q);
+                const float4 v = *reinterpret_cast<const float4 *>(As + (size_t)k * TR_BM + ty * RPT + q);
                 a[q] = v.x;
                 a[q + 1] = v.y;
                 a[q + 2] = v.z;
                 a[q + 3] = v.w;
             } else {
-                const double2 v = *reinterpret_cast<const double2 *>(As + (size_t)k * TR_BM + ty * 8 + q);
+                const double2 v = *reinterpret_cast<const double2 *>(As + (size_t)k * TR_BM + ty * RPT + q);
                 a[q] = v.x;
                 a[q + 1] = v.y;
             }
@@ -1613,15 +1613,15 @@ __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, 
 #pragma unroll
         for (int c = 0; c < CPT; ++c) b[c] = Bs[(size_t)(tx + NTX * c) * ldb + k];
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
+        for (int r = 0; r < RPT; ++r)
 #pragma unroll
             for (int c = 0; c < CPT; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < RPT; ++r)
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) Cs[(tx + NTX * c) * (TR_BM + 1) + ty * 8 + r] = acc[r][c];
+        for (int c = 0; c < CPT; ++c) Cs[(tx + NTX * c) * (TR_BM + 1) + ty * RPT + r] = acc[r][c];
     __syncthreads();
     const int warp = tid >> 5, lane = tid & 31;
     const int rows = min(TR_BM, nc - rb);
@@ -1632,14 +1632,14 @@ __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, 
     }
 }
 
-template <class T, int BN, int NTH, int BM>
+template <class T, int BN, int NTH, int BM, int RPT>
 __global__ void __launch_bounds__(NTH)
 k_tree_translate(const T *__restrict__ ops, int nc, int cs, int ldb, const int4 *__restrict__ chunks,
                  const int *__restrict__ p_out, const int *__restrict__ p_in, const T *__restrict__ in,
                  T *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_in[BN], s_out[BN];
-    tree_translate_block<T, BN, NTH, BM>(ops, nc, cs, ldb, chunks[blockIdx.x], blockIdx.y * BM, p_out, p_in, in, out,
+    tree_translate_block<T, BN, NTH, BM, RPT>(ops, nc, cs, ldb, chunks[blockIdx.x], blockIdx.y * BM, p_out, p_in, in, out,
                                          smraw, s_in, s_out);
 }
 
@@ -1648,7 +1648,8 @@ template <class T>
 static int tree_ldb(int cs) {
     return (int)(((cs * sizeof(T) + 127) / 128 * 128 + 16) / sizeof(T));
 }
-constexpr int TREE_BM = 64;  // operator rows per CTA (two CTAs per chunk at p = 10)
+constexpr int TREE_BM = 32;  // operator rows per CTA (four CTAs per chunk at p = 10)
+constexpr int TREE_RPT = 4;  // rows per thread
 template <class T>
 static size_t tree_translate_smem(int nc, int cs) {
     const size_t ab = ((size_t)nc * TREE_BM + (size_t)TR_BN_TREE * tree_ldb<T>(cs)) * sizeof(T);
@@ -1927,6 +1928,29 @@ static void ev_rec(Mesh &m, bool timed, int k) {
     if (timed && m.tm.on) BEM_CUDA(cudaEventRecord(m.tm.ev[k], m.stream));
 }
 
+// The expansions that a pass accumulates into (multipoles above the leaf
+// level, locals from level 2) and the tensor-core M2L's work counter, cleared
+// by one kernel ahead of P2M: three memsets in the chain of launches kept
+// each of the kernels after them from starting early.
+__global__ void k_clear(float4 *a, int64_t na, float4 *b, int64_t nb, int *counter) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < na) a[i] = z;
+    if (i < nb) b[i] = z;
+    if (i == 0) *counter = 0;
+}
+
+template <class T>
+static void clear_expansions(Mesh &m, const Tree &t, T *M, T *L, int cs) {
+    // rows are multiples of 16 bytes (cs is a multiple of 4)
+    const int64_t rm = t.L >= 3 ? t.lvl_off[t.L] - t.lvl_off[2] : 0, rl = t.ncell - t.lvl_off[2];
+    const int64_t w = (int64_t)cs * sizeof(T) / sizeof(float4), n = std::max<int64_t>(1, std::max(rm, rl) * w);
+    k_clear<<<cdiv(n, 256), 256, 0, m.stream>>>(reinterpret_cast<float4 *>(M + (size_t)t.lvl_off[2] * cs), rm * w,
+                                                reinterpret_cast<float4 *>(L + (size_t)t.lvl_off[2] * cs), rl * w,
+                                                m.dev_err.p + 1);
+    BEM_CHECK_LAUNCH();
+}
+
 // one level of M2M or L2L: the chunks [chunk0, chunk0 + nchunk) of the
 // grouped tree translations
 template <class T>
@@ -1937,7 +1961,7 @@ static void tree_translate(const T *ops, int nc, int cs, int rblocks, const Tree
     const size_t sm = tree_translate_smem<T>(nc, cs);
     if (sm <= TREE_SMEM_MAX) {
         dim3 gt(nchunk, cdiv(nc, TREE_BM));
-        auto kern = k_tree_translate<T, TR_BN_TREE, TR_THREADS_TREE, TREE_BM>;
+        auto kern = k_tree_translate<T, TR_BN_TREE, TR_THREADS_TREE, TREE_BM, TREE_RPT>;
         set_smem<T>(kern, sm);
         // programmatic dependent launch: the CTAs may start while the previous
         // kernel of the stream finishes (the kernel waits before it reads its
@@ -2054,15 +2078,11 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
         if (!t.p2p_hdr[wk].p) throw Error(BEM_ECUDA, "near field: work list missing");
         const P2PList wl{t.p2p_hdr[wk].p, t.p2p_rec[wk].p};
         auto go = [&](auto k128, auto k256) {
-            if (small) {
-                constexpr size_t sm = p2p_smem<T, 128>();
-                if (sm + 9216 > 48 * 1024) ensure_smem_attr(reinterpret_cast<const void *>(k128), sm);
-                k128<<<t.nleaf, 128, sm, ss>>>(wl, trec, nrec, strec, hh, near_b, ntab);
-            } else {
-                constexpr size_t sm = p2p_smem<T, 256>();
-                if (sm + 9216 > 48 * 1024) ensure_smem_attr(reinterpret_cast<const void *>(k256), sm);
-                k256<<<t.nleaf, 256, sm, ss>>>(wl, trec, nrec, strec, hh, near_b, ntab);
-            }
+            const int nt = small ? 128 : 256;
+            const size_t sm = small ? p2p_smem<T, 128>() : p2p_smem<T, 256>();
+            auto k = small ? k128 : k256;
+            if (sm + 9216 > 48 * 1024) ensure_smem_attr(reinterpret_cast<const void *>(k), sm);
+            k<<<t.nleaf, nt, sm, ss>>>(wl, trec, nrec, strec, hh, near_b, ntab);
         };
         const bool wide = t.ws == 2;
         if (t.ws != 1 && t.ws != 2) throw Error(BEM_EUNSUPPORTED, "near field: separation not built");
@@ -2086,19 +2106,21 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
         BEM_CHECK_LAUNCH();
         if (tn) BEM_CUDA(cudaEventRecord(m.tm.nev[2], ss));
     };
-    // The near field forks off after the upward sweep (P2M, M2M): the M2L
-    // kernel holds every SM by itself (one CTA with ~225 KB of shared memory
-    // each) and runs first at the highest priority, and the near field's CTAs
-    // fill the SMs around the latency-bound launches before and after it.
-    // Measured on the 81,920-panel product: 0.312 ms forked here, 0.319 ms
-    // forked before P2M, 0.339 ms after M2L, 0.342 ms one after the other.
-    auto fork_near = [&]() {
+    // The near field runs beside the far field on its own low-priority stream,
+    // from the pass's start: its CTAs fill the SMs around P2M (bound by HBM) and
+    // the M2M levels (bound by latency), whose CTAs fit into what one near-field
+    // CTA leaves (k_tree_translate: 128 threads, 33 KB).  The tensor-core M2L
+    // needs whole SMs and follows the last of them.  Measured on the
+    // 81,920-panel product: 0.256 ms; 0.276 forked after the upward sweep,
+    // 0.272 in two parts, the second released once M2L holds the SMs.  (While
+    // the tree kernels took 63 KB and 256 threads a CTA they waited for three
+    // near-field CTAs of one SM to end at once: 0.279 ms forked at the start.)
+    if (conc) {
         BEM_CUDA(cudaEventRecord(m.ev_fork, s));
         BEM_CUDA(cudaStreamWaitEvent(m.stream2, m.ev_fork, 0));
         launch_near(m.stream2);
         BEM_CUDA(cudaEventRecord(m.ev_join, m.stream2));
-    };
-    if (conc && !far) fork_near();
+    }
     if (far) {
         T *M = B::M(m), *L = B::L(m);
         const int cs = cell_stride(p);
@@ -2106,14 +2128,12 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
         const int rblocks = cdiv(nc, TR_BM);
         const size_t trsm = translate_smem<T, TR_BN_M2L>();
         if (dense) set_smem<T>(k_translate<T, TR_BN_M2L, TR_THREADS>, trsm);
+        if (dense) clear_expansions<T>(m, t, M, L, cs);
         // P2M
         p2m_leaves<T>(tv, t.nleaf, sk, srec, qpanel, dens, p, cs, inv_h, M, s);
         ev_rec(m, timed, 1);
         // M2M: parents at levels L-1 .. 2
         if (dense) {
-            if (t.L >= 3)
-                BEM_CUDA(cudaMemsetAsync(M + (size_t)t.lvl_off[2] * cs, 0,
-                                         (size_t)(t.lvl_off[t.L] - t.lvl_off[2]) * cs * sizeof(T), s));
             tree_sweep<T>(m, B::Om2m(tb), nc, cs, t, true, M, M, s);
         } else {
             const size_t sm = 2 * (size_t)(p + 1) * W * sizeof(cpx<T>);
@@ -2125,7 +2145,6 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
             }
         }
         ev_rec(m, timed, 2);
-        if (conc) fork_near();
         // M2L: every cell at levels 2..L
         if (dense) {
             m2l_dense<T>(m, t, B::Om2l(tb), nc, cs, rblocks, trsm, M, L, timed);
@@ -2461,15 +2480,13 @@ void build_near_table(Mesh &m, const double *panels) {
 template <class T>
 static void m2l_dense(Mesh &m, const Tree &t, const T *Oop, int nc, int cs, int rblocks, size_t trsm,
                       T *M, T *L, bool timed) {
-    // L at levels >= 2 = the M2L sums (cleared first unless written whole)
+    // L at levels >= 2 += the M2L sums
     if constexpr (std::is_same<T, float>::value) {
         if (use_tc_m2l(m)) {
             m2l_tc(m, t, M, L, timed);
             return;
         }
     }
-    BEM_CUDA(cudaMemsetAsync(L + (size_t)t.lvl_off[2] * cs, 0, (size_t)(t.ncell - t.lvl_off[2]) * cs * sizeof(T),
-                             m.stream));
     if (t.m2l_nchunk == 0) return;
     dim3 g(t.m2l_nchunk, rblocks);
     k_translate<T, TR_BN_M2L, TR_THREADS><<<g, TR_THREADS, trsm, m.stream>>>(Oop, nc, cs, t.g_chunk.p + t.m2l_chunk0,
@@ -2539,6 +2556,7 @@ static void run_pass_t(Mesh &m, const double *lam, double *out) {
         const int rblocks = cdiv(nc, TR_BM);
         const size_t trsm = translate_smem<T, TR_BN_M2L>();
         set_smem<T>(k_translate<T, TR_BN_M2L, TR_THREADS>, trsm);
+        clear_expansions<T>(m, t, M, L, cs);
         {
             const int th = std::max(32, p2m_threads(p, sizeof(T)));
             const size_t sm = (size_t)th * nc * sizeof(T);
@@ -2546,9 +2564,6 @@ static void run_pass_t(Mesh &m, const double *lam, double *out) {
             k_p2m_dipole<T><<<t.nleaf, th, sm, s>>>(tv, dbeg, drec, dnrm, dlam, p, cs, inv_h, M);
             BEM_CHECK_LAUNCH();
         }
-        if (t.L >= 3)
-            BEM_CUDA(cudaMemsetAsync(M + (size_t)t.lvl_off[2] * cs, 0,
-                                     (size_t)(t.lvl_off[t.L] - t.lvl_off[2]) * cs * sizeof(T), s));
         tree_sweep<T>(m, B::Om2m(tb), nc, cs, t, true, M, M, s);
         m2l_dense<T>(m, t, B::Om2l(tb), nc, cs, rblocks, trsm, M, L);
         tree_sweep<T>(m, B::Ol2l(tb), nc, cs, t, false, L, L, s);

@@ -231,7 +231,7 @@ struct Timers {
     bool near_before_l2p = false;
     cudaEvent_t ev[8] = {};
     double ms[7] = {};
-    cudaEvent_t kev[4] = {};  // inside the tensor-core M2L stage: split | kernel | (unused)
+    cudaEvent_t kev[4] = {};  // inside the tensor-core M2L stage: (unused) | kernel | (unused)
     cudaEvent_t nev[3] = {};  // inside the near-field phase: strength records | near-field kernel
 };
 
@@ -320,7 +320,6 @@ struct Mesh {
     DArray<double> far_d, near_d;      // (fp64 mode)
     DArray<double> io_a, io_b;         // staging for host or unsorted arguments
     DArray<double> red;                // reduction scratch
-    DArray<float> Mtc;                 // multipoles split hi|lo for the tensor-core M2L
     DArray<float> dpart_f;             // direct-sum partials (mixed)
     DArray<double> dpart_d;            // direct-sum partials (fp64)
     DArray<float4> dsrc;               // direct-sum source records of one segment (mixed)
@@ -342,8 +341,9 @@ struct Mesh {
 
 // --------------------------------------------------------------- helpers
 inline int ncoef(int p) { return (p + 1) * (p + 1); }
-// per-cell stride of the expansion arrays: (p+1)^2 rounded up to 4 values
-inline int cell_stride(int p) { return ((p + 1) * (p + 1) + 3) & ~3; }
+// per-cell stride of the expansion arrays: (p+1)^2 rounded up to 32 values, so
+// that rows start on whole 128-byte lines
+inline int cell_stride(int p) { return ((p + 1) * (p + 1) + 31) & ~31; }
 inline int cdiv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // geometry + trees (bem_tree.cu)
@@ -404,7 +404,6 @@ __host__ __device__ inline int tc_table_index(int in, int out) {
 void build_tc_super(Tree &t, const std::vector<int4> &chunks_m2l, cudaStream_t s);
 void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed = false);
 bool use_tc_m2l(const Mesh &m);
-size_t tc_staging_floats(const Mesh &m);
 void compute_bbox(const double *d, int64_t n, int stride, double *lo, double *hi, cudaStream_t s);
 
 // fast multipole passes (bem_fmm.cu).  `dens` is indexed in sorted panel

@@ -10,8 +10,8 @@
 // products).  The operator (A) and the accumulators live in tensor memory;
 // the multipoles (B) are staged in shared memory one K-block (32
 // coefficients, 128 bytes of a row) at a time in the K-major layout with the
-// 128-byte swizzle, so that a warp's copy instruction reads four whole
-// 128-byte rows from global memory.  A persistent, warp-specialised kernel
+// 128-byte swizzle: a warp's load reads four 128-byte pieces of rows from
+// global memory in FP32 and the producers split them as they store.  A persistent, warp-specialised kernel
 // runs the pairs of one class as a stream of 128-pair tiles (producers, one
 // MMA thread, epilogue; see k_m2l_tc).  The epilogue adds each pair's
 // local-expansion row into its target cell with vector reductions
@@ -61,10 +61,15 @@ __device__ __forceinline__ uint64_t tc_desc_sw128(uint32_t saddr) {
 constexpr uint32_t TC_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
                               ((uint32_t)(128 >> 4) << 24);
 
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
+// x as the sum of two TF32 values (11 significant bits each): h the nearest,
+// in integer arithmetic (ties away from zero), l the rest rounded by Dekker's
+// splitting (ties to even).  Both run on the ALU and FMA pipes, which this
+// kernel leaves idle.  A NaN or infinity leaves l NaN.
+__device__ __forceinline__ void split_tf32(float x, uint32_t &h, uint32_t &l) {
+    h = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    const float r = x - __uint_as_float(h);
+    const float c = __fmul_rn(r, 8193.f);  // 2^13 + 1
+    l = __float_as_uint(__fsub_rn(c, __fsub_rn(c, r)));
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t phase) {
@@ -109,9 +114,9 @@ constexpr int TC_ND = 2;                       // TMEM accumulators of TC_BN col
 constexpr int TC_RING = 16;                    // work items in flight between the roles
 constexpr int TC_WARP_MMA = 0;                 // lane 0 issues the MMAs
 constexpr int TC_WARP_EPI0 = 1;                // warps 1..4: epilogue (TMEM lane quadrant = warp % 4)
-constexpr int TC_WARP_PROD0 = 5;               // warps 5..8: copies of B, operator into TMEM
-constexpr int TC_NPROD = 4 * 32, TC_NEPI = 4 * 32;
-constexpr int TC_THREADS = 9 * 32;
+constexpr int TC_WARP_PROD0 = 5;               // warps 5..12: staging of B, operator into TMEM
+constexpr int TC_NPROD = 8 * 32, TC_NEPI = 4 * 32;
+constexpr int TC_THREADS = 13 * 32;
 constexpr int TC_ROWS_PER_PROD = TC_BN * 8 / TC_NPROD;  // rows of a stage per producer thread (8 granules each)
 
 __device__ __forceinline__ void bulk_prefetch_l2(const void *g, uint32_t bytes) {
@@ -121,30 +126,36 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void *g, uint32_t bytes) 
 // The persistent kernel: one CTA per SM takes work items (offset class,
 // first pair, number of pairs: up to 8 tiles of 128 pairs) from a global
 // counter, largest first.  Tiles are numbered continuously across a CTA's
-// items and each tile passes through TC_NKB stages (one per K-block), so the
-// pipeline never drains between items:
-//  * producers (warps 5-8): the leader fetches the next item, publishes it
+// items and each tile passes through nkb stages (one per K-block of 32
+// coefficients: 4 at p = 10, 2 at p = 6), so the pipeline never drains between
+// items:
+//  * producers (warps 5-12): the leader fetches the next item, publishes it
 //    in a shared ring (mbarrier itemFull) and prefetches its operator into
-//    L2; all 128 copy the K-block of the tile's split multipoles into stage
-//    g % TC_NS (cp.async: a warp instruction moves four 128-byte rows,
-//    written in the 128-byte swizzle; mbarrier fullB).  After the first tile
-//    of an item they wait for the last MMA of the previous item (its fullD
-//    commit) and write the item's operator into tensor memory (aReady),
-//    split from FP32 into its TF32 hi and lo parts on the way.
+//    L2; all 256 hold a whole tile of multipoles in registers (FP32, 4 rows x
+//    16 bytes per K-block and thread): each K-block is split into its TF32 hi
+//    and lo parts and stored to stage g % TC_NS in the 128-byte swizzle
+//    (mbarrier fullB), and its registers are loaded with the next tile's
+//    K-block at once, a tile of time ahead.  After the first tile of an item
+//    they wait for the last MMA of the previous item (its fullD commit) and
+//    write the item's operator into tensor memory (aReady), split the same way.
 //  * MMA (warp 0, lane 0): per item waits aReady; per tile waits a free
-//    accumulator (emptyD), per K-block its stage (fullB), issues 4 K-steps x
+//    accumulator (emptyD), per K-block its stage (fullB), issues its K-steps x
 //    3 products with A from tensor memory and commits to emptyB; after the
 //    last K-block it commits to fullD.
 //  * epilogue (warps 1-4): reads its TMEM lane quadrant, frees the
 //    accumulator, transposes the tile into shared memory rows (one local
-//    expansion row of cs floats per pair), then the 128 threads add the rows
-//    into their target cells of `out`, four coefficients per reduction.
+//    expansion row of cs floats per pair), then each warp adds whole rows into
+//    their target cells of `out`, four coefficients per lane and reduction.
+// What bounded it: the copies of B.  Multipoles split beforehand are 1 KB a
+// pair, 128 KB a tile, 5.4k cycles at the 24 B/cycle an SM's copies reach,
+// against 3.2k cycles of MMAs; FP32 rows are 64 KB and need no split kernel.
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_m2l_tc(const float *__restrict__ A_all,
          const int4 *__restrict__ items, int nitems, int *__restrict__ next_item,
-         const int *__restrict__ p_out, const int *__restrict__ p_in, int cs,
-         const float *__restrict__ Mtc, float *__restrict__ out, int *__restrict__ err,
+         const int *__restrict__ p_out, const int *__restrict__ p_in, int nc, int cs,
+         const float *__restrict__ M, float *__restrict__ out, int *__restrict__ err,
          long long budget) {
+    const int nkb = (nc + TC_KB - 1) / TC_KB;  // K-blocks that hold coefficients
     extern __shared__ __align__(1024) unsigned char smraw[];
     // 1024-byte aligned base (the 128-byte swizzle repeats every 1024 B)
     unsigned char *sm = smraw + ((1024u - (smem_u32(smraw) & 1023u)) & 1023u);
@@ -176,17 +187,16 @@ k_m2l_tc(const float *__restrict__ A_all,
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tm = s_tmem;
-    // launched as a programmatic dependent of the multipole split: the set-up
-    // above overlaps it; the split multipoles, the cleared local expansions
-    // and the work counter are read only after this wait
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (An ordinary launch: as a programmatic dependent of the last M2M level its
+    // CTAs would hold their SMs, idle, until that level ends: 8 uneven
+    // molecules at once 10.17 against 10.57 ms.)
     int ntile_done = 0;  // tiles whose MMAs were all issued (MMA thread)
     int nstage_done = 0; // K-block stages whose MMAs were issued and committed (MMA thread)
 
     if (warp >= TC_WARP_PROD0) {
         // ---------------- producers
         const int ptid = tid - TC_WARP_PROD0 * 32;
-        const int pw = ptid >> 5;                            // producer warp 0..3
+        const int pw = ptid >> 5;                            // producer warp 0..7
         const int quad = warp & 3, row = 32 * quad + lane;  // TMEM lane of this thread
         const int gq = lane & 7, r4 = lane >> 3;            // 16-byte granule, row within a group of 4
         // every wait is made warp-uniform (__all_sync) and every item starts with
@@ -215,42 +225,66 @@ k_m2l_tc(const float *__restrict__ A_all,
             const int4 sc = s_item[slot];
             if (sc.x < 0) break;
             const int ntl = (sc.z + TC_BN - 1) / TC_BN;
-            // source cells of the tile rows this thread copies: n = 32 pw + 4 v + r4
+            // source cells of the tile rows this thread stages
             auto load_srcs = [&](int c, int *dst) {
-                const int y = sc.y + TC_BN * c, z = min(TC_BN, sc.z - TC_BN * c);
+                const int y = sc.y + TC_BN * c, z = min(TC_BN, sc.z - TC_BN * c);  // z <= 0 past the item
 #pragma unroll
-                for (int v = 0; v < TC_ROWS_PER_PROD; ++v) {
-                    const int n = 32 * pw + 4 * v + r4;
-                    dst[v] = (n < z) ? p_in[y + n] : -1;
+                for (int i = 0; i < TC_ROWS_PER_PROD; ++i) {
+                    const int n = 4 * TC_ROWS_PER_PROD * pw + 4 * i + r4;
+                    dst[i] = (n < z) ? p_in[y + n] : -1;
                 }
             };
-            int srcs[TC_ROWS_PER_PROD], nxt[TC_ROWS_PER_PROD];
-            load_srcs(0, srcs);
+            // K-block kb of the tile whose source cells are src, FP32; zero beyond
+            // the coefficients (a row's padding is not initialised)
+            float4 v[TC_NKB][TC_ROWS_PER_PROD];
+            auto load_kb = [&](int kb, const int *src) {
+                const int k0 = TC_KB * kb + 4 * gq;
+#pragma unroll
+                for (int i = 0; i < TC_ROWS_PER_PROD; ++i) {
+                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (src[i] >= 0 && k0 < nc) x = __ldcg(reinterpret_cast<const float4 *>(M + (size_t)src[i] * cs + k0));
+                    v[kb][i] = x;
+                }
+            };
+            int nxt[TC_ROWS_PER_PROD];
+            load_srcs(0, nxt);
+#pragma unroll
+            for (int kb = 0; kb < TC_NKB; ++kb) load_kb(kb, nxt);
+            load_srcs(1, nxt);
             for (int c = 0; c < ntl; ++c, ++t) {
-                if (c + 1 < ntl) load_srcs(c + 1, nxt);
-                for (int kb = 0; kb < TC_NKB && !fail; ++kb) {
-                    const int g = TC_NKB * t + kb;
+#pragma unroll
+                for (int kb = 0; kb < TC_NKB; ++kb) {
+                    if (kb >= nkb || fail) continue;
+                    const int g = nkb * t + kb;
                     const int st = g % TC_NS, k = g / TC_NS;
                     const bool okB = __all_sync(0xffffffffu, k < 1 || mbar_wait_bounded(smem_u32(&emptyB[st]),
                                                                                        (uint32_t)((k - 1) & 1), budget));
                     if (!okB) {
                         atomicExch(err, 1);
                         fail = true;
-                        break;
+                        continue;
                     }
-                    const uint32_t bh = sbase + (uint32_t)(st * TC_STAGE_BYTES);
-                    const uint32_t bl = bh + TC_BN * TC_KB * 4;
+                    unsigned char *bh = sm + (size_t)st * TC_STAGE_BYTES, *bl = bh + TC_BN * TC_KB * 4;
+                    const int left = nc - (TC_KB * kb + 4 * gq);  // coefficients from this granule on
 #pragma unroll
-                    for (int v = 0; v < TC_ROWS_PER_PROD; ++v) {
-                        const int n = 32 * pw + 4 * v + r4;
-                        const int src = srcs[v];
-                        const float *gsrc = Mtc + (size_t)(src >= 0 ? src : 0) * 2 * TC_K + TC_KB * kb + 4 * gq;
-                        const uint32_t nb = src >= 0 ? 16u : 0u;  // 0: zero-fill (padding rows)
+                    for (int i = 0; i < TC_ROWS_PER_PROD; ++i) {
+                        const int n = 4 * TC_ROWS_PER_PROD * pw + 4 * i + r4;
+                        const float x[4] = {v[kb][i].x, left > 1 ? v[kb][i].y : 0.f, left > 2 ? v[kb][i].z : 0.f,
+                                            left > 3 ? v[kb][i].w : 0.f};
+                        uint4 h, l;
+                        split_tf32(x[0], h.x, l.x);
+                        split_tf32(x[1], h.y, l.y);
+                        split_tf32(x[2], h.z, l.z);
+                        split_tf32(x[3], h.w, l.w);
                         const uint32_t off = (uint32_t)(n * 128 + ((gq ^ (n & 7)) << 4));
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(bh + off), "l"(gsrc), "r"(nb));
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(bl + off), "l"(gsrc + TC_K), "r"(nb));
+                        *reinterpret_cast<uint4 *>(bh + off) = h;
+                        *reinterpret_cast<uint4 *>(bl + off) = l;
                     }
-                    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&fullB[st])) : "memory");
+                    // the stage was written through the generic proxy: order it before
+                    // the tensor core's (async proxy) reads
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    mbar_arrive(smem_u32(&fullB[st]));
+                    if (c > 0 && c + 1 < ntl) load_kb(kb, nxt);
                 }
                 if (fail) break;
                 if (c == 0) {
@@ -266,48 +300,45 @@ k_m2l_tc(const float *__restrict__ A_all,
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;");
                     // operator layout [k / 4][row][k % 4]: the warp's rows read 512
-                    // contiguous bytes per load; 32 coefficients at a time, each
+                    // contiguous bytes per load; 16 coefficients at a time, each
                     // split into its TF32 hi part and the TF32 rest (the 3xTF32
                     // operands) and stored to both halves of the operator's columns
                     const float4 *ga = reinterpret_cast<const float4 *>(A_all + (size_t)sc.x * TC_K * TC_K) + row;
-#pragma unroll 1
-                    for (int part = 0; part < 4; ++part) {
-                        const float4 *gp = ga + part * 8 * TC_K;
-                        uint32_t vh[32], vl[32];
+#pragma unroll 2
+                    for (int part = pw >> 2; part < 2 * nkb; part += 2) {  // two warps per lane quadrant
+                        const float4 *gp = ga + part * 4 * TC_K;
+                        uint32_t vh[16], vl[16];
 #pragma unroll
-                        for (int q = 0; q < 32; q += 4) {
+                        for (int q = 0; q < 16; q += 4) {
                             const float4 f = __ldg(gp + (q >> 2) * TC_K);
                             const float x[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                vh[q + e] = to_tf32(x[e]);
-                                vl[q + e] = to_tf32(x[e] - __uint_as_float(vh[q + e]));
-                            }
+                            for (int e = 0; e < 4; ++e) split_tf32(x[e], vh[q + e], vl[q + e]);
                         }
 #pragma unroll
                         for (int hl = 0; hl < 2; ++hl) {
-                            const uint32_t *v = hl ? vl : vh;
+                            const uint32_t *w = hl ? vl : vh;
                             asm volatile(
-                                "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-                                "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(
-                                    tm + ((uint32_t)(32 * quad) << 16) + (uint32_t)(hl ? TC_A_LO : TC_A_HI) +
-                                    (uint32_t)(32 * part)),
-                                "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
-                                "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]),
-                                "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]),
-                                "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
-                                "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]));
+                                "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+                                "%15,%16};" ::"r"(tm + ((uint32_t)(32 * quad) << 16) +
+                                                  (uint32_t)(hl ? TC_A_LO : TC_A_HI) + (uint32_t)(16 * part)),
+                                "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]),
+                                "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]),
+                                "r"(w[15]));
                         }
                     }
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;");
                     mbar_arrive(smem_u32(&aReady));
-                }
+                    // the second tile: its latency passes under the first tile's MMAs
+                    if (ntl > 1) {
 #pragma unroll
-                for (int v = 0; v < TC_ROWS_PER_PROD; ++v) srcs[v] = nxt[v];
+                        for (int kb = 0; kb < TC_NKB; ++kb) load_kb(kb, nxt);
+                    }
+                }
+                load_srcs(c + 2, nxt);  // needed after the next tile's first stage
             }
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp == TC_WARP_MMA) {
         // ---------------- MMA issue (one thread)
         if (lane == 0) {
@@ -335,17 +366,14 @@ k_m2l_tc(const float *__restrict__ A_all,
                         break;
                     }
                     const uint32_t dt = tm + (uint32_t)(TC_D0 + d * TC_BN);
-                    for (int kb = 0; kb < TC_NKB; ++kb) {
-                        const int g = TC_NKB * t + kb;
+                    for (int kb = 0; kb < nkb; ++kb) {
+                        const int g = nkb * t + kb;
                         const int st = g % TC_NS, k = g / TC_NS;
                         if (!mbar_wait_bounded(smem_u32(&fullB[st]), (uint32_t)(k & 1), budget)) {
                             atomicExch(err, 1);
                             fail = true;
                             break;
                         }
-                        // the stage was written by cp.async (generic proxy): order it before
-                        // the tensor core's (async proxy) reads
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::after_thread_sync;");
                         const uint32_t bh = sbase + (uint32_t)(st * TC_STAGE_BYTES);
                         const uint32_t bl = bh + TC_BN * TC_KB * 4;
@@ -375,7 +403,6 @@ k_m2l_tc(const float *__restrict__ A_all,
         const int quad = warp & 3;
         const int row = 32 * quad + lane;
         const int etid = tid - TC_WARP_EPI0 * 32;  // 0 .. TC_NEPI - 1
-        __shared__ int s_tgt[TC_BN];               // target cells of the tile's pairs
         bool fail = false;
         int t = 0;
         for (int i = 0; !fail; ++i) {
@@ -408,11 +435,12 @@ k_m2l_tc(const float *__restrict__ A_all,
                     fail = true;
                     break;
                 }
-                // every thread has left the previous tile's reductions (Ct, s_tgt free)
+                // the previous tile's reductions have read Ct
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 asm volatile("bar.sync 1, %0;" ::"n"(TC_NEPI) : "memory");
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 const int y = sc.y + TC_BN * c, z = min(TC_BN, sc.z - TC_BN * c);
-                if (etid < z) s_tgt[etid] = p_out[y + etid];
+                const int tgt = etid < z ? p_out[y + etid] : -1;
 #pragma unroll 1
                 for (int cg = 0; cg < TC_BN; cg += 32) {
                     uint32_t r[32];
@@ -433,19 +461,18 @@ k_m2l_tc(const float *__restrict__ A_all,
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;");
                 mbar_arrive(smem_u32(&emptyD[d]));
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("bar.sync 1, %0;" ::"n"(TC_NEPI) : "memory");
-                // every pair's row added into its target cell, four coefficients per
-                // vector reduction, spread over the epilogue threads
-                const int q4 = cs >> 2;
-                for (int idx = etid; idx < z * q4; idx += TC_NEPI) {
-                    const int j = idx / q4, q = idx - j * q4;
-                    const float4 v = *reinterpret_cast<const float4 *>(Ct + j * cs + 4 * q);
-                    asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(out + (size_t)s_tgt[j] * cs + 4 * q),
-                                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                // every pair's row added into its target cell by one bulk reduction
+                if (tgt >= 0)
+                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(
+                                     out + (size_t)tgt * cs),
+                                 "r"(smem_u32(Ct + etid * cs)), "r"((nc + 3) / 4 * 16)
                                  : "memory");
-                }
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         }
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     // before the CTA's shared memory and tensor memory go away, every commit
     // arrival must have landed: the MMA thread waits (bounded) for the last
@@ -499,52 +526,18 @@ void build_tc_super(Tree &t, const std::vector<int4> &chunks_m2l, cudaStream_t s
     BEM_CUDA(cudaStreamSynchronize(s));
 }
 
-// hi/lo TF32 split of the multipoles of the M2L sources (cells of levels
-// >= 2), rows of 2 x 128 floats: hi | lo, zero beyond (p+1)^2.  One thread
-// per 4 coefficients of a cell (16-byte loads and stores; cs is a multiple
-// of 4, and a group at or past cs is not read).
-__global__ void k_split_m(const float *M, int first, int ncell, int nc, int cs, float *Mtc) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the M2L kernel may start its set-up
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t c = first + (i >> 5);
-    const int k0 = 4 * (int)(i & 31);
-    if (c >= ncell) return;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k0 < cs) x = *reinterpret_cast<const float4 *>(M + c * cs + k0);
-    float v[4] = {x.x, x.y, x.z, x.w};
-    float h[4], l[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        if (k0 + e >= nc) v[e] = 0.f;
-        const uint32_t t = to_tf32(v[e]);
-        h[e] = __uint_as_float(t);
-        l[e] = __uint_as_float(to_tf32(v[e] - h[e]));
-    }
-    float *row = Mtc + c * 2 * TC_K;
-    *reinterpret_cast<float4 *>(row + k0) = make_float4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<float4 *>(row + TC_K + k0) = make_float4(l[0], l[1], l[2], l[3]);
-}
-
-// L (levels >= 2) = sum over the M2L pairs of T_o M_s: L cleared, the
-// multipoles split hi | lo, then the persistent kernel adds every pair's row
-// into its target.
+// L (levels >= 2, cleared by the pass) += sum over the M2L pairs of T_o M_s.
 void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed) {
     const Tables &tb = tables_for(m, t);
     const int nc = (m.opt.p + 1) * (m.opt.p + 1);
     const int cs = cell_stride(m.opt.p);
-    const int first = t.lvl_off[2];
-    BEM_CUDA(cudaMemsetAsync(L + (size_t)first * cs, 0, (size_t)(t.ncell - first) * cs * sizeof(float), m.stream));
     if (t.tc_nsuper == 0) return;
-    if (m.Mtc.n < (size_t)t.ncell * 2 * TC_K) throw Error(BEM_ECUDA, "tensor-core staging buffer too small");
     const bool tk = timed && m.tm.on && m.tm.kev[0];
     auto kev = [&](int k) {
         if (tk) BEM_CUDA(cudaEventRecord(m.tm.kev[k], m.stream));
     };
-    BEM_CUDA(cudaMemsetAsync(m.dev_err.p + 1, 0, sizeof(int), m.stream));  // work-item counter
     kev(0);
     if (cs % 4 != 0) throw Error(BEM_ECUDA, "tensor-core staging: cell stride not a multiple of 4");
-    k_split_m<<<cdiv((int64_t)(t.ncell - first) * 32, 256), 256, 0, m.stream>>>(M, first, t.ncell, nc, cs, m.Mtc.p);
-    BEM_CHECK_LAUNCH();
     const size_t sm = tc_smem_bytes();
     int dev = 0, nsm = 0;
     BEM_CUDA(cudaGetDevice(&dev));
@@ -552,35 +545,11 @@ void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed) {
     const int grid = std::max(1, std::min(t.tc_nsuper, nsm));
     kev(1);
     ensure_smem_attr(reinterpret_cast<const void *>(k_m2l_tc), sm);
-    {
-        // programmatic dependent launch after the split (the kernel waits
-        // before it reads anything the split or earlier work wrote)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(TC_THREADS);
-        cfg.dynamicSmemBytes = sm;
-        cfg.stream = m.stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const float *A = tb.Tc_f.p;
-        const int4 *items = t.tc_super.p;
-        const int nitems = t.tc_nsuper;
-        int *counter = m.dev_err.p + 1, *err = m.dev_err.p;
-        const int *po = t.g_out.p, *pi = t.g_in.p;
-        const float *Mtc = m.Mtc.p;
-        const long long budget = m.wait_budget;
-        BEM_CUDA(cudaLaunchKernelEx(&cfg, k_m2l_tc, A, items, nitems, counter, po, pi, cs, Mtc, L, err, budget));
-    }
+    k_m2l_tc<<<grid, TC_THREADS, sm, m.stream>>>(tb.Tc_f.p, t.tc_super.p, t.tc_nsuper, m.dev_err.p + 1, t.g_out.p,
+                                                 t.g_in.p, nc, cs, M, L, m.dev_err.p, m.wait_budget);
+    BEM_CHECK_LAUNCH();
     kev(2);
     kev(3);
 }
-
-size_t tc_staging_floats(const Mesh &m) {
-    return (size_t)std::max(m.tp.ncell, m.tc.ncell) * 2 * TC_K;
-}
-
 
 }  // namespace bem

@@ -44,3 +44,29 @@ def test_highest_order_against_oracle(pkg):
     x = P.bq()
     with pkg.Mesh(m.panels, m.charges, m.eps_in, m.eps_out, precision=pkg.BEM_FP64, p=16, depth=3) as g:
         close(g.matvec(torch.from_numpy(x).cuda()).cpu().numpy(), P.A(x), 1e-6, what="p = 16")
+
+
+@pytest.mark.parametrize("p", [1, 4, 5, 6, 7, 8, 9, 10])
+def test_tensor_core_m2l_orders(pkg, p):
+    """Every number of K-blocks of the tensor-core M2L (32 coefficients each,
+    the last one ragged) against the dense FP32 form: products kept to 2^-21
+    by the split on one side and FP32 sums of up to 121 terms on both."""
+    m = synth.small_molecule(4)
+    x = torch.from_numpy(np.random.default_rng(p).standard_normal(m.n_p)).cuda()
+    y = []
+    for mode in (pkg.BEM_M2L_TC, pkg.BEM_M2L_DENSE):
+        with pkg.Mesh(m.panels, m.charges, m.eps_in, m.eps_out, p=p, depth=3, m2l_mode=mode,
+                      flags=pkg.BEM_FLAG_NO_NEAR) as g:
+            y.append((g.matvec(x) - x).cpu().numpy())
+    close(y[0], y[1], 4e-6, what="far field")
+
+
+def test_tensor_core_m2l_keeps_nan_and_infinity(pkg):
+    m = synth.small_molecule(4)
+    with pkg.Mesh(m.panels, m.charges, m.eps_in, m.eps_out, depth=3) as g:
+        for bad in (float("nan"), float("inf")):
+            x = torch.ones(m.n_p, dtype=torch.float64, device="cuda")
+            x[7] = bad
+            # every panel lies in the near or the far field of panel 7
+            assert not torch.isfinite(g.matvec(x)).any()
+        assert torch.isfinite(g.matvec(torch.ones_like(x))).all()
