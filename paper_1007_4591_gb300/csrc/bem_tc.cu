@@ -136,19 +136,26 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void *g, uint32_t bytes) 
 //    and lo parts and stored to stage g % TC_NS in the 128-byte swizzle
 //    (mbarrier fullB), and its registers are loaded with the next tile's
 //    K-block at once, a tile of time ahead.  After the first tile of an item
-//    they wait for the last MMA of the previous item (its fullD commit) and
-//    write the item's operator into tensor memory (aReady), split the same way.
+//    they wait for the last MMA of the previous item (aFree) and write the
+//    item's operator into tensor memory (aReady), split the same way.  (A
+//    barrier of its own: a parity wait must not run two phases ahead, and with
+//    one K-block a tile the producers are several tiles ahead of fullD.)
 //  * MMA (warp 0, lane 0): per item waits aReady; per tile waits a free
 //    accumulator (emptyD), per K-block its stage (fullB), issues its K-steps x
 //    3 products with A from tensor memory and commits to emptyB; after the
-//    last K-block it commits to fullD.
+//    last K-block it commits to fullD, after an item's last tile to aFree.
 //  * epilogue (warps 1-4): reads its TMEM lane quadrant, frees the
 //    accumulator, transposes the tile into shared memory rows (one local
-//    expansion row of cs floats per pair), then each warp adds whole rows into
-//    their target cells of `out`, four coefficients per lane and reduction.
-// What bounded it: the copies of B.  Multipoles split beforehand are 1 KB a
-// pair, 128 KB a tile, 5.4k cycles at the 24 B/cycle an SM's copies reach,
-// against 3.2k cycles of MMAs; FP32 rows are 64 KB and need no split kernel.
+//    expansion row of cs floats per pair), then adds every row into its target
+//    cell of `out` by one bulk reduction.
+// What bounds it, on 2.7M pairs (81,920-panel molecules, 27 of them; 461 us, 6.7k
+// cycles a tile): nothing alone.  Without the reductions 424, operator writes
+// 428, two of the three MMAs 395, stores to the stages 371, with nothing but
+// the MMAs 348 us: the MMAs issue at 106 cycles each (5.1k a tile).  Multipoles
+// split beforehand (1 KB a pair, copied) took 514 us and a split kernel;
+// reductions by vector instructions 512.  An FP16 split in three products with
+// scaled operands, half the MMAs, took 479: the tiles then wait for copies and
+// reductions, 128 KB of L2 traffic each.
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_m2l_tc(const float *__restrict__ A_all,
          const int4 *__restrict__ items, int nitems, int *__restrict__ next_item,
@@ -162,7 +169,7 @@ k_m2l_tc(const float *__restrict__ A_all,
     const uint32_t sbase = smem_u32(sm);
     float *Ct = reinterpret_cast<float *>(sm + (size_t)TC_NS * TC_STAGE_BYTES);  // [TC_BN][cs]
     __shared__ __align__(8) uint64_t fullB[TC_NS], emptyB[TC_NS], fullD[TC_ND], emptyD[TC_ND];
-    __shared__ __align__(8) uint64_t aReady, itemFull[TC_RING];
+    __shared__ __align__(8) uint64_t aReady, aFree, itemFull[TC_RING];
     __shared__ int4 s_item[TC_RING];
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -181,6 +188,7 @@ k_m2l_tc(const float *__restrict__ A_all,
             mbar_init(smem_u32(&emptyD[i]), TC_NEPI);
         }
         mbar_init(smem_u32(&aReady), TC_NPROD);
+        mbar_init(smem_u32(&aFree), 1);
         for (int i = 0; i < TC_RING; ++i) mbar_init(smem_u32(&itemFull[i]), 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -191,6 +199,7 @@ k_m2l_tc(const float *__restrict__ A_all,
     // CTAs would hold their SMs, idle, until that level ends: 8 uneven
     // molecules at once 10.17 against 10.57 ms.)
     int ntile_done = 0;  // tiles whose MMAs were all issued (MMA thread)
+    int nitem_done = 0;  // items whose MMAs were all issued (MMA thread)
     int nstage_done = 0; // K-block stages whose MMAs were issued and committed (MMA thread)
 
     if (warp >= TC_WARP_PROD0) {
@@ -290,9 +299,8 @@ k_m2l_tc(const float *__restrict__ A_all,
                 if (c == 0) {
                     // the item's operator into tensor memory, once the previous
                     // item's MMAs (which read the old one) have completed
-                    const int tp = t - 1;
-                    const bool okA = __all_sync(0xffffffffu, t < 1 || mbar_wait_bounded(smem_u32(&fullD[tp % TC_ND]),
-                                                                                       (uint32_t)((tp / TC_ND) & 1), budget));
+                    const bool okA = __all_sync(0xffffffffu, i < 1 || mbar_wait_bounded(smem_u32(&aFree),
+                                                                                       (uint32_t)((i - 1) & 1), budget));
                     if (!okA) {
                         atomicExch(err, 1);
                         fail = true;
@@ -394,7 +402,12 @@ k_m2l_tc(const float *__restrict__ A_all,
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                      smem_u32(&fullD[d]))
                                  : "memory");
+                    if (c == ntl - 1)  // the item's MMAs all issued: its operator is free when they end
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                         smem_u32(&aFree))
+                                     : "memory");
                 }
+                if (!fail) nitem_done = i + 1;
             }
             ntile_done = t;
         }
@@ -478,7 +491,7 @@ k_m2l_tc(const float *__restrict__ A_all,
     // arrival must have landed: the MMA thread waits (bounded) for the last
     // completion of each B stage (which follows all MMAs issued before it,
     // also those of a tile left unfinished by a failed wait) and of the last
-    // accumulator
+    // accumulator and operator release
     if (warp == TC_WARP_MMA && lane == 0 && nstage_done > 0) {
         const int ng = nstage_done;
         for (int st = 0; st < TC_NS && st < ng; ++st) {
@@ -489,6 +502,7 @@ k_m2l_tc(const float *__restrict__ A_all,
             const int t = ntile_done - 1;
             mbar_wait_bounded(smem_u32(&fullD[t % TC_ND]), (uint32_t)((t / TC_ND) & 1));
         }
+        if (nitem_done > 0) mbar_wait_bounded(smem_u32(&aFree), (uint32_t)((nitem_done - 1) & 1));
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();

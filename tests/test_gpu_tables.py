@@ -70,3 +70,17 @@ def test_tensor_core_m2l_keeps_nan_and_infinity(pkg):
             # every panel lies in the near or the far field of panel 7
             assert not torch.isfinite(g.matvec(x)).any()
         assert torch.isfinite(g.matvec(torch.ones_like(x))).all()
+
+
+@pytest.mark.parametrize("p", [2, 4, 6, 10])
+def test_tensor_core_m2l_many_items(pkg, p):
+    """Hundreds of offset classes and thousands of tiles, where the kernel's
+    producers run ahead of its MMAs (by tiles and items at low orders)."""
+    m = synth.globular(6)
+    x = torch.from_numpy(np.random.default_rng(p).uniform(0.5, 1.5, m.n_p)).cuda()
+    y = []
+    for mode in (pkg.BEM_M2L_TC, pkg.BEM_M2L_DENSE):
+        with pkg.Mesh(m.panels, np.zeros((0, 4)), m.eps_in, m.eps_out, p=p, leaf_size=32, m2l_mode=mode,
+                      flags=pkg.BEM_FLAG_NO_NEAR) as g:
+            y.append((g.matvec(x) - x).cpu().numpy())
+    close(y[0], y[1], 4e-6, what="far field")
