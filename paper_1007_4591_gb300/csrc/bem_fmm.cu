@@ -71,9 +71,16 @@ __device__ __forceinline__ float ex2a(float x) {
     return y;
 }
 __device__ __forceinline__ float rinv3(float r2) { return ex2a(-1.5f * lg2a(r2)); }
+// FP64: the hardware's 20-bit estimate y of r^-1 (relative error d, |d| < 2^-20)
+// corrected by the binomial series of (1 - e)^(-3/2) in e = 1 - r^2 y^2 up to e^2
+// (the next term is below 2^-56): six FP64 operations where rsqrt and its cube
+// take eight.  FP64 issue bounds every caller (a pair takes 20.2 issue slots
+// against 21.4), and the error falls from 5.4e-16 to 2.3e-16.
 __device__ __forceinline__ double rinv3(double r2) {
-    const double ri = rsqrt(r2);
-    return ri * ri * ri;
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    const double y2 = y * y, e = fma(-r2, y2, 1.0), y3 = y * y2;
+    return fma(y3 * e, fma(e, 1.875, 1.5), y3);
 }
 
 // Regular solid harmonics R_n^m(x,y,z), 0 <= m <= n <= p, handed to emit(n, m, re, im).
@@ -467,9 +474,9 @@ template <> struct Pk<double> {
 // Targets per thread: 3 in FP32 (measured against 4: the product 0.2883 vs
 // 0.2947 ms, no register spills at 64 registers, and leaves of ~17 targets
 // pad to 18 instead of 20), 2 in FP64.
-template <class T> struct P2PTpt;
-template <> struct P2PTpt<float> { static constexpr int v = 3; };
-template <> struct P2PTpt<double> { static constexpr int v = 2; };
+// (The Galerkin targets, seven to a panel, fill groups of 4 and hide latency
+// with three CTAs of 256 threads per SM: 32,000 panels 0.336 -> 0.297 ms.)
+template <class T, int TGT> struct P2PTpt { static constexpr int v = sizeof(T) == 8 ? 2 : (TGT == TGT_QUAD_DN ? 4 : 3); };
 // Pair slots per thread and tile: FP32 tiles of 384 pairs for 128 threads
 // (24 KB for the two buffers: 8 CTAs per SM) and 512 for 256 threads.
 template <class T, int NT> struct P2PPpt { static constexpr int v = 1; };
@@ -550,14 +557,14 @@ struct NearTab {
 // NB: the most neighbour leaves a leaf has (27 for one-cell separation, 125
 // for the charge tree's two cells).
 template <class T, int SRC, int TGT, int NT, int NB = 27>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 1024 / NT : 1)
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (TGT == TGT_QUAD_DN ? 896 : 1024) / NT : 1)
 k_p2p(P2PList wl, const typename V4T<T>::t *tgt, const typename V4T<T>::t *nrm,
       const typename V4T<T>::t *src, T h, T *out, NearTab tab) {
     using V4 = typename V4T<T>::t;
     using P = Pk<T>;
     using v2 = typename P::v;
     static_assert(NB <= NT, "one thread per neighbour leaf in the set-up");
-    constexpr int P2P_TPT = P2PTpt<T>::v;
+    constexpr int P2P_TPT = P2PTpt<T, TGT>::v;
     constexpr int PPT = P2PPpt<T, NT>::v;
     constexpr int TP = NT * PPT;                 // pair slots per buffer
     constexpr int NCP = (int)(sizeof(V4) / 16);  // 16-byte copies per record
