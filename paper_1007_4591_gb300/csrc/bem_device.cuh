@@ -110,6 +110,11 @@ template <class T>
 void p2m_leaves(const TreeView &tv, int nleaf, SrcKind sk, const typename V4T<T>::t *src, const int *qpanel,
                 const double *dens, int p, int cs, T inv_h, T *M, cudaStream_t s);
 
+// P2M of dipoles lam_i nrm_i at rec_i, dbeg the leaves' CSR (p in 1..MAXP).
+template <class T>
+void p2m_dipoles(const TreeView &tv, int nleaf, const int *dbeg, const typename V4T<T>::t *rec,
+                 const typename V4T<T>::t *nrm, const double *lam, int p, int cs, T inv_h, T *M, cudaStream_t s);
+
 // L2P of every leaf with a compile-time expansion order (p in {6, 8, 10,
 // 12}); one CTA of nth threads per leaf, queued on `s`.  Returns false (and
 // launches nothing) for other orders.  With epi.y set (collocation targets)

@@ -769,75 +769,6 @@ k_p2p(P2PList wl, const typename V4T<T>::t *tgt, const typename V4T<T>::t *nrm,
 }
 
 // ------------------------------------------------------ transposed K' pass
-// Dipole sources p_i = lam_i n_i at the collocation points.  The multipole
-// of a dipole is its own degree-1 expansion D_1^0 = p_z,
-// D_1^{+-1} = -+ (p_x -+ i p_y)/2 translated like an M2M:
-//   M_n^m = sum_{l=-1..1} conj(R_{n-1}^{m-l}(c - z)) D_1^l,
-// accumulated here while the recurrence emits R_k^l (scaled by 1/h).
-template <class T>
-__global__ void k_p2m_dipole(TreeView tv, const int *dbeg, const typename V4T<T>::t *rec,
-                             const typename V4T<T>::t *nrm, const double *lam, int p, int cs,
-                             T inv_h, T *M) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    T *sh = reinterpret_cast<T *>(smraw);
-    const int leaf = blockIdx.x;
-    const int b = dbeg[leaf], e = dbeg[leaf + 1];
-    const int nc = (p + 1) * (p + 1);
-    constexpr int MAXACC = 10;
-    T acc[MAXACC];
-#pragma unroll
-    for (int k = 0; k < MAXACC; ++k) acc[k] = 0;
-    for (int base = b; base < e; base += blockDim.x) {
-        const int i = base + threadIdx.x;
-        T *row = sh + threadIdx.x * nc;
-        for (int c = 0; c < nc; ++c) row[c] = 0;
-        if (i < e) {
-            const typename V4T<T>::t r = rec[i], nv = nrm[i];
-            const T l = (T)lam[i] * inv_h;
-            const T px = l * nv.x, py = l * nv.y, pz = l * nv.z;
-            // D_1^0 = pz, D_1^1 = -(px - i py)/2, D_1^-1 = (px + i py)/2
-            const T d1r = -px / 2, d1i = py / 2, dmr = px / 2, dmi = py / 2;
-            regular_solid<T>(r.x * inv_h, r.y * inv_h, r.z * inv_h, p - 1, [&](int k, int l, T re, T im) {
-                const int n = k + 1;
-                // conj(R) = (re, -im); add conj(R) * D to M_n^m
-                auto add = [&](int m, T dr, T di) {  // m >= 0
-                    const T vr = re * dr + im * di, vi = re * di - im * dr;
-                    if (m == 0) row[n * n] += vr;
-                    else {
-                        row[n * n + 2 * m - 1] += vr;
-                        row[n * n + 2 * m] += vi;
-                    }
-                };
-                add(l, pz, 0);
-                add(l + 1, d1r, d1i);
-                if (l >= 1) add(l - 1, dmr, dmi);
-                if (l == 1) {
-                    // R_k^{-1} = -conj(R_k^1): conj(R_k^{-1}) D_1^1 = -(re + i im)(d1r + i d1i)
-                    row[n * n] += -(re * d1r - im * d1i);
-                }
-            });
-        }
-        __syncthreads();
-        const int cnt = min((int)blockDim.x, e - base);
-        int k = 0;
-        for (int c = threadIdx.x; c < nc; c += blockDim.x, ++k) {
-            T a = 0;
-            for (int j = 0; j < cnt; ++j) a += sh[j * nc + c];
-#pragma unroll
-            for (int q = 0; q < MAXACC; ++q)
-                if (q == k) acc[q] += a;
-        }
-        __syncthreads();
-    }
-    T *out = M + (size_t)(tv.leaf0 + leaf) * cs;
-    int k = 0;
-    for (int c = threadIdx.x; c < nc; c += blockDim.x, ++k) {
-#pragma unroll
-        for (int q = 0; q < MAXACC; ++q)
-            if (q == k) out[c] = acc[q];
-    }
-}
-
 // Near field of the transposed product, organised like the forward kernel:
 // one CTA per leaf T of collocation points; the quadrature points of the
 // adjacent leaves are moved into T's frame exactly as the forward kernel
@@ -1918,13 +1849,6 @@ static int l2p_threads(int64_t ntgt, int nleaf) {
     return (int)std::min<int64_t>(128, std::max<int64_t>(32, (avg + 31) / 32 * 32));
 }
 
-static int p2m_threads(int p, size_t elt) {
-    const size_t nc = (size_t)(p + 1) * (p + 1);
-    int t = 128;
-    while (t > 32 && (size_t)t * nc * elt > 96 * 1024) t >>= 1;
-    return t;
-}
-
 template <class T, class KernelT>
 static void set_smem(KernelT kern, size_t bytes) {
     if (bytes > 48 * 1024) ensure_smem_attr(reinterpret_cast<const void *>(kern), bytes);
@@ -2564,13 +2488,7 @@ static void run_pass_t(Mesh &m, const double *lam, double *out) {
         const size_t trsm = translate_smem<T, TR_BN_M2L>();
         set_smem<T>(k_translate<T, TR_BN_M2L, TR_THREADS>, trsm);
         clear_expansions<T>(m, t, M, L, cs);
-        {
-            const int th = std::max(32, p2m_threads(p, sizeof(T)));
-            const size_t sm = (size_t)th * nc * sizeof(T);
-            set_smem<T>(k_p2m_dipole<T>, sm);
-            k_p2m_dipole<T><<<t.nleaf, th, sm, s>>>(tv, dbeg, drec, dnrm, dlam, p, cs, inv_h, M);
-            BEM_CHECK_LAUNCH();
-        }
+        p2m_dipoles<T>(tv, t.nleaf, dbeg, drec, dnrm, dlam, p, cs, inv_h, M, s);
         tree_sweep<T>(m, B::Om2m(tb), nc, cs, t, true, M, M, s);
         m2l_dense<T>(m, t, B::Om2l(tb), nc, cs, rblocks, trsm, M, L);
         tree_sweep<T>(m, B::Ol2l(tb), nc, cs, t, false, L, L, s);
