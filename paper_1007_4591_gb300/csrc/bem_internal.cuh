@@ -152,8 +152,20 @@ struct Tree {
     // M2M pairs (out = parent, in = child) and L2L pairs (out = child,
     // in = parent) per child level, sorted by the child's octant.  A chunk is
     // (operator, first pair, pair count <= 64, 0).
-    DArray<int> g_out, g_in;      // all grouped pairs: M2L, then M2M and L2L per level
-    DArray<int4> g_chunk;
+    DArray<int> g_out, g_in;      // grouped tree pairs: M2M and L2L per level
+    DArray<int4> g_chunk;         // their chunks
+    // M2L pairs by what a pass moves: any pair; charges to panels (the source
+    // cell holds charges, the target cell panels); panels to charges.  The
+    // other pairs of a charge tree carry zero multipoles or unread locals.
+    struct M2LPairs {
+        DArray<int> out, in;
+        DArray<int4> chunk;       // (operator, first pair, pair count <= 64, 0)
+        int nchunk = 0;
+        DArray<int4> super;       // tensor-core M2L work items (operator, first pair, pairs)
+        int nsuper = 0;
+        size_t bytes() const { return out.bytes() + in.bytes() + chunk.bytes() + super.bytes(); }
+    } m2l[3];
+    enum { M2L_ALL = 0, M2L_CHG_TO_PANEL = 1, M2L_PANEL_TO_CHG = 2 };
     DArray<int> p2p_order;        // leaves by decreasing near-field work (launch order)
     // near-field work lists in launch order, per source kind (quadrature
     // points, charges): two int4 of leaf data and nb records per CTA
@@ -170,9 +182,6 @@ struct Tree {
     DArray<float> p2m_seg_f;      // [nseg x cell stride] moments (mixed precision)
     DArray<double> p2m_seg_d;     // [nseg x cell stride] moments (FP64)
     int p2m_seg_p = -1;           // expansion order of the moments (-1: none built)
-    DArray<int4> tc_super;        // tensor-core M2L work items (offset, first chunk, chunks)
-    int tc_nsuper = 0;
-    int m2l_chunk0 = 0, m2l_nchunk = 0;
     std::vector<int> m2m_chunk0, m2m_nchunk, l2l_chunk0, l2l_nchunk; // indexed by child level
     size_t bytes() const;
 };
@@ -401,8 +410,8 @@ constexpr int TC_TABLE_DIM = 128;
 __host__ __device__ inline int tc_table_index(int in, int out) {
     return ((in >> 2) * TC_TABLE_DIM + out) * 4 + (in & 3);
 }
-void build_tc_super(Tree &t, const std::vector<int4> &chunks_m2l, cudaStream_t s);
-void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed = false);
+void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cudaStream_t s);
+void m2l_tc(Mesh &m, const Tree &t, const Tree::M2LPairs &g, const float *M, float *L, bool timed = false);
 bool use_tc_m2l(const Mesh &m);
 void compute_bbox(const double *d, int64_t n, int stride, double *lo, double *hi, cudaStream_t s);
 

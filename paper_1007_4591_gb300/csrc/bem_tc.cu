@@ -522,7 +522,7 @@ size_t tc_smem_bytes() { return 1024 + (size_t)TC_NS * TC_STAGE_BYTES + (size_t)
 // Work items of the persistent kernel: (offset class, first pair, number of
 // pairs), up to TC_CHUNKS_PER_ITEM consecutive 64-pair chunks of one class
 // (tiles of 128 pairs), largest first.
-void build_tc_super(Tree &t, const std::vector<int4> &chunks_m2l, cudaStream_t s) {
+void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cudaStream_t s) {
     std::vector<int4> sup;
     int i = 0;
     const int n = (int)chunks_m2l.size();
@@ -533,19 +533,19 @@ void build_tc_super(Tree &t, const std::vector<int4> &chunks_m2l, cudaStream_t s
         i = j;
     }
     std::stable_sort(sup.begin(), sup.end(), [](const int4 &a, const int4 &b) { return a.z > b.z; });
-    t.tc_super.alloc(sup.size());
-    t.tc_nsuper = (int)sup.size();
+    g.super.alloc(sup.size());
+    g.nsuper = (int)sup.size();
     if (!sup.empty())
-        BEM_CUDA(cudaMemcpyAsync(t.tc_super.p, sup.data(), sup.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+        BEM_CUDA(cudaMemcpyAsync(g.super.p, sup.data(), sup.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
     BEM_CUDA(cudaStreamSynchronize(s));
 }
 
 // L (levels >= 2, cleared by the pass) += sum over the M2L pairs of T_o M_s.
-void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed) {
+void m2l_tc(Mesh &m, const Tree &t, const Tree::M2LPairs &g, const float *M, float *L, bool timed) {
     const Tables &tb = tables_for(m, t);
     const int nc = (m.opt.p + 1) * (m.opt.p + 1);
     const int cs = cell_stride(m.opt.p);
-    if (t.tc_nsuper == 0) return;
+    if (g.nsuper == 0) return;
     const bool tk = timed && m.tm.on && m.tm.kev[0];
     auto kev = [&](int k) {
         if (tk) BEM_CUDA(cudaEventRecord(m.tm.kev[k], m.stream));
@@ -556,11 +556,11 @@ void m2l_tc(Mesh &m, const Tree &t, const float *M, float *L, bool timed) {
     int dev = 0, nsm = 0;
     BEM_CUDA(cudaGetDevice(&dev));
     BEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int grid = std::max(1, std::min(t.tc_nsuper, nsm));
+    const int grid = std::max(1, std::min(g.nsuper, nsm));
     kev(1);
     ensure_smem_attr(reinterpret_cast<const void *>(k_m2l_tc), sm);
-    k_m2l_tc<<<grid, TC_THREADS, sm, m.stream>>>(tb.Tc_f.p, t.tc_super.p, t.tc_nsuper, m.dev_err.p + 1, t.g_out.p,
-                                                 t.g_in.p, nc, cs, M, L, m.dev_err.p, m.wait_budget);
+    k_m2l_tc<<<grid, TC_THREADS, sm, m.stream>>>(tb.Tc_f.p, g.super.p, g.nsuper, m.dev_err.p + 1, g.out.p,
+                                                 g.in.p, nc, cs, M, L, m.dev_err.p, m.wait_budget);
     BEM_CHECK_LAUNCH();
     kev(2);
     kev(3);

@@ -648,7 +648,7 @@ static void build_tree(Mesh &m, Tree &t, SetKeys cen, SetKeys qp, SetKeys chg, i
 }
 
 size_t Tree::bytes() const {
-    return g_out.bytes() + g_in.bytes() + g_chunk.bytes() + p2p_order.bytes() + tc_super.bytes() +
+    return g_out.bytes() + g_in.bytes() + g_chunk.bytes() + p2p_order.bytes() + m2l[0].bytes() + m2l[1].bytes() + m2l[2].bytes() +
            p2p_hdr[0].bytes() + p2p_hdr[1].bytes() + p2p_rec[0].bytes() + p2p_rec[1].bytes() +
            key.bytes() + ijk.bytes() + parent.bytes() + child_beg.bytes() + child_end.bytes() +
            cen_beg.bytes() + qp_beg.bytes() + chg_beg.bytes() + nbr_off.bytes() + nbr.bytes() +
