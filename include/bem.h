@@ -75,7 +75,7 @@ extern "C" {
                                      angles; checked when n_c x n_p x 7 <= 4e10, skipped above) */
 #define BEM_FLAG_M2L_REDUCE 16u   /* accepted for compatibility, no effect: the tensor-core M2L
                                      always adds each pair's row into its target cell with
-                                     vector reductions (no per-pair buffer) */
+                                     bulk reductions (no per-pair buffer) */
 #define BEM_FLAG_CHARGE_NEAR_EXACT 32u /* higher-accuracy panel integration of the charges
                                      (Sec. 2.1): in C s, C^T q and grad_x C s every pair of a
                                      charge and a panel whose centroid lies within 2.5 sqrt(A_j)
@@ -188,7 +188,7 @@ int bem_mesh_create(const double *panels, int64_t n_p, const double *charges, in
 int bem_mesh_destroy(bem_mesh *mesh);
 
 /* Replace the point charges (same or different count); the panel tree is kept,
- * the charge tree and lists and C^T q are rebuilt.  charges [n_c][4] f64. */
+ * C^T q and, where the charge sums use one, the charge tree are rebuilt.  charges [n_c][4] f64. */
 int bem_set_charges(bem_mesh *mesh, const double *charges, int64_t n_c);
 
 /* y = A x = x + Ehat K' x  (the BEM operator of Eq. ASC), x, y [n_p] f64.

@@ -14,10 +14,9 @@
 // global memory in FP32 and the producers split them as they store.  A persistent, warp-specialised kernel
 // runs the pairs of one class as a stream of 128-pair tiles (producers, one
 // MMA thread, epilogue; see k_m2l_tc).  The epilogue adds each pair's
-// local-expansion row into its target cell with vector reductions
-// (red.global.add.v4.f32): the targets' local expansions (a few MB) stay in
-// L2, which absorbs the reductions at about the rate HBM would take the rows
-// (measured 4.9 TB/s against 5.5 TB/s for plain stores), and no per-pair
+// local-expansion row into its target cell with a bulk reduction
+// (cp.reduce.async.bulk, add.f32): the targets' local expansions (a few MB)
+// stay in L2, which absorbs the reductions, and no per-pair
 // buffer is written or read back.  Every wait is bounded: the pipeline waits by
 // the mesh's wait budget (bem_set_wait_budget), after which the kernel
 // raises an error flag; the last wait for its own MMAs (always about a
