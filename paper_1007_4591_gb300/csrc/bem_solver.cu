@@ -6,6 +6,7 @@
 // Givens rotations for the least-squares update, one 8-byte residual written to
 // pinned host memory per iteration to decide convergence.
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "bem_internal.cuh"
@@ -142,14 +143,25 @@ void matvec_sorted(Mesh &m, const double *xs, double *ys) {
 
 // --------------------------------------------------------------- BLAS-1
 // Reductions end in the kernel that starts them: the last CTA to arrive
-// (a ticket that wraps to zero) adds the CTAs' parts in a fixed order.  At
-// GMRES sizes these kernels are launches and latency, not bandwidth (8 n bytes
-// a vector, 0.1 us at 81,920 panels): an Arnoldi step was 11 launches and a
-// copy, is four launches, and the host reads the residual from pinned memory
-// the device writes (81,920 panels, 8 iterations: solve 2.98 -> 2.75 ms; 1,280 panels 0.88 -> 0.70).
+// (a ticket that wraps to zero) adds the CTAs' parts in a fixed order.  Up to
+// some 100,000 panels these kernels are launches and latency, not bandwidth
+// (8 n bytes a vector, 0.1 us at 81,920 panels): an Arnoldi step was 11 launches
+// and a copy, is four launches, and the host reads the residual from pinned
+// memory the device writes.  Above, FP64 issue and the passes over the basis
+// count: the second pass of Gram-Schmidt subtracts and forms its products in
+// one.  Kernels of a step, averages of 7 to 10 steps, against the eleven:
+// 81,920 panels 38 us (60), 655,360 74 us (92), 2.6M 0.170 ms (0.208), 12.3M
+// 0.640 ms (0.778).
 
-// rows of a CTA: a multiple of its threads, at most one CTA per SM
-static int rows_for(int64_t n) { return RED_THREADS * std::max(1, cdiv(n, (int64_t)RED_THREADS * 152)); }
+// CTAs of a reduction over n rows, each a stride of the grid apart so that the
+// CTAs sweep a vector together: 152 while the vectors lie in L2 and the end of
+// the reduction costs more than a sparse sweep (655,360 rows: 74 us with 152,
+// 77 with 304), from 24 rows a thread on twice as many (1.3M rows 115 and 104
+// us, 12.3M 0.942 and 0.640 ms; 608: 119 us and 0.652 ms).
+static int ctas_for(int64_t n) {
+    const int64_t most = n < (int64_t)152 * RED_THREADS * 24 ? 152 : 304;
+    return (int)std::min<int64_t>(cdiv(n, RED_THREADS), most);
+}
 
 __device__ __forceinline__ bool last_cta(unsigned *ticket) {
     __shared__ bool last;
@@ -161,36 +173,71 @@ __device__ __forceinline__ bool last_cta(unsigned *ticket) {
     return last;
 }
 
-// part[i][CTA] = the CTA's rows' share of V_i . w, for nvec vectors, 8 at a time
-__device__ __forceinline__ void dot_rows(const double *V, size_t ld, int nvec, const double *w, int64_t b, int64_t e,
-                                         double *part) {
-    __shared__ double sh[8][RED_THREADS / 32];
+// nvec vectors are `full` blocks of VEC_BLOCK and a last one of NV (1 to
+// VEC_BLOCK), a compile-time parameter (MORE: full > 0): FP64 issue bounds these kernels once
+// they fill the chip, and a lane that a predicate turns off takes its slot all
+// the same.  A thread has the loads of a whole block in flight.
+constexpr int VEC_BLOCK = 8;
+
+// part[i][CTA] = the CTA's sum of s[i]
+template <int NV>
+__device__ __forceinline__ void cta_parts(double (&s)[NV], double *part) {
+    __shared__ double sh[NV][RED_THREADS / 32];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    for (int i0 = 0; i0 < nvec; i0 += 8) {
-        const int ni = min(8, nvec - i0);
-        double s[8];
+    __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] = 0.0;
-        for (int64_t r = b + threadIdx.x; r < e; r += RED_THREADS) {
-            const double x = w[r];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (i < ni) s[i] += V[(size_t)(i0 + i) * ld + r] * x;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            if (i < ni)
-                for (int o = 16; o > 0; o >>= 1) s[i] += __shfl_down_sync(0xffffffffu, s[i], o);
-            if (lane == 0) sh[i][wp] = s[i];
-        }
-        __syncthreads();
-        if (threadIdx.x < ni) {
-            double t = 0.0;
-            for (int k = 0; k < RED_THREADS / 32; ++k) t += sh[threadIdx.x][k];
-            part[(size_t)(i0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
-        }
+    for (int i = 0; i < NV; ++i) {
+        for (int o = 16; o > 0; o >>= 1) s[i] += __shfl_down_sync(0xffffffffu, s[i], o);
+        if (lane == 0) sh[i][wp] = s[i];
     }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double t = 0.0;
+        for (int k = 0; k < RED_THREADS / 32; ++k) t += sh[threadIdx.x][k];
+        part[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = t;
+    }
+}
+
+// sum_i h[i] V_i[r] over `full` blocks and the last one, whose values are v
+template <int NV, bool MORE>
+__device__ __forceinline__ double row_sum(const double *__restrict__ V, size_t ld, int full, const double *h, int64_t r,
+                                          const double (&v)[NV]) {
+    double a = 0.0;
+    for (int i0 = 0; MORE && i0 < VEC_BLOCK * full; i0 += VEC_BLOCK) {
+        double u[VEC_BLOCK];
+#pragma unroll
+        for (int i = 0; i < VEC_BLOCK; ++i) u[i] = V[(size_t)(i0 + i) * ld + r];
+#pragma unroll
+        for (int i = 0; i < VEC_BLOCK; ++i) a += h[i0 + i] * u[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) a += h[(MORE ? VEC_BLOCK * full : 0) + i] * v[i];
+    return a;
+}
+
+// part[i][CTA] = the CTA's rows' share of (last block)_i . w; with SUB,
+// w -= sum_i h[i] V_i over all blocks first, in the same pass
+template <int NV, bool SUB, bool MORE>
+__device__ __forceinline__ void dot_block(const double *__restrict__ V, size_t ld, int full, const double *h,
+                                          double *__restrict__ w, int64_t n, double *part) {
+    constexpr int U = NV >= 5 ? 1 : (NV >= 3 ? 2 : 4);  // rows of a thread in flight
+    const double *__restrict__ Vl = V + (size_t)VEC_BLOCK * full * ld;
+    double s[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) s[i] = 0.0;
+#pragma unroll U
+    for (int64_t r = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; r < n; r += (int64_t)gridDim.x * RED_THREADS) {
+        double v[NV], x = w[r];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = Vl[(size_t)i * ld + r];
+        if (SUB) {
+            x -= row_sum<NV, MORE>(V, ld, full, h, r, v);
+            w[r] = x;
+        }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) s[i] += v[i] * x;
+    }
+    cta_parts<NV>(s, part + (size_t)VEC_BLOCK * full * gridDim.x);
 }
 
 // out[i] = the sum of vector i's parts (a warp per vector)
@@ -204,22 +251,11 @@ __device__ __forceinline__ void sum_parts(const double *part, int nvec, double *
     }
 }
 
-// w -= sum_i h[i] V_i over the CTA's rows
-__device__ __forceinline__ void sub_rows(const double *V, size_t ld, int nvec, const double *h, double *w, int64_t b,
-                                         int64_t e) {
-    for (int64_t r = b + threadIdx.x; r < e; r += RED_THREADS) {
-        double a = 0.0;
-        for (int i = 0; i < nvec; ++i) a += h[i] * V[(size_t)i * ld + r];
-        w[r] -= a;
-    }
-}
-
 // out[0] = V . w (mode 0) or its square root (mode 1), also written to `host`
 __global__ void __launch_bounds__(RED_THREADS)
-k_dot(const double *V, const double *w, int64_t n, int rows, double *part, unsigned *ticket, int mode, double *out,
+k_dot(const double *V, const double *w, int64_t n, double *part, unsigned *ticket, int mode, double *out,
       volatile double *host) {
-    const int64_t b = (int64_t)blockIdx.x * rows, e = min(n, b + rows);
-    dot_rows(V, 0, 1, w, b, e, part);
+    dot_block<1, false, false>(V, 0, 0, nullptr, const_cast<double *>(w), n, part);  // reads w only
     if (!last_cta(ticket)) return;
     __shared__ double t;
     sum_parts(part, 1, &t);
@@ -231,15 +267,16 @@ k_dot(const double *V, const double *w, int64_t n, int rows, double *part, unsig
     }
 }
 
-// First pass of classical Gram-Schmidt, h = V^T w, or (hsub set) the second:
+// First pass of classical Gram-Schmidt, h = V^T w, or (SUB) the second:
 // w -= V hsub, then h = V^T w.
-__global__ void __launch_bounds__(RED_THREADS)
-k_cgs(const double *V, size_t ld, int nvec, const double *hsub, double *w, int64_t n, int rows, double *part,
+template <int NV, bool SUB, bool MORE>
+__global__ void __launch_bounds__(RED_THREADS, MORE ? 3 : 4)
+k_cgs(const double *V, size_t ld, int full, const double *hsub, double *w, int64_t n, double *part,
       unsigned *ticket, double *h) {
-    const int64_t b = (int64_t)blockIdx.x * rows, e = min(n, b + rows);
-    if (hsub) sub_rows(V, ld, nvec, hsub, w, b, e);
-    dot_rows(V, ld, nvec, w, b, e, part);
-    if (last_cta(ticket)) sum_parts(part, nvec, h);
+    // every thread reads back the rows it writes
+    dot_block<NV, SUB, MORE>(V, ld, full, hsub, w, n, part);
+    for (int f = 0; MORE && f < full; ++f) dot_block<VEC_BLOCK, false, false>(V, ld, f, nullptr, w, n, part);  // block f
+    if (last_cta(ticket)) sum_parts(part, VEC_BLOCK * full + NV, h);
 }
 
 // Givens update of Hessenberg column j (column-major, leading dimension m1).
@@ -271,13 +308,26 @@ __device__ void givens(double *H, int m1, const double *hcol, int j, double *cs,
 
 // The Arnoldi step's end: w -= V h2, |w|, the Hessenberg column h + h2 | |w|
 // through the Givens rotations, the residual to the host.
-__global__ void __launch_bounds__(RED_THREADS)
-k_cgs_end(const double *V, size_t ld, int j, double *h, const double *h2, double *w, int64_t n, int rows, double *part,
+template <int NV, bool MORE>
+__global__ void __launch_bounds__(RED_THREADS, MORE ? 3 : 4)
+k_cgs_end(const double *V, size_t ld, int full, double *h, const double *h2, double *w, int64_t n, double *part,
           unsigned *ticket, double *H, int m1, double *cs, double *sn, double *g, double inv_bnorm, double *out,
           volatile double *host) {
-    const int64_t b = (int64_t)blockIdx.x * rows, e = min(n, b + rows);
-    sub_rows(V, ld, j + 1, h2, w, b, e);
-    dot_rows(w, 0, 1, w, b, e, part);
+    constexpr int U = NV >= 5 ? 1 : (NV >= 3 ? 2 : 4);
+    const int j = VEC_BLOCK * full + NV - 1;
+    const double *__restrict__ Vl = V + (size_t)VEC_BLOCK * full * ld;
+    double *__restrict__ wr = w;
+    double s[1] = {0.0};
+#pragma unroll U
+    for (int64_t r = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; r < n; r += (int64_t)gridDim.x * RED_THREADS) {
+        double v[NV], x = wr[r];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = Vl[(size_t)i * ld + r];
+        x -= row_sum<NV, MORE>(V, ld, full, h2, r, v);
+        wr[r] = x;
+        s[0] += x * x;
+    }
+    cta_parts<1>(s, part);
     if (!last_cta(ticket)) return;
     __shared__ double t;
     sum_parts(part, 1, &t);
@@ -338,14 +388,24 @@ __global__ void k_backsolve(const double *H, int m1, const double *g, int k, dou
 
 // V . w (mode 0) or its square root (mode 1), left in *out and read by the host
 static double dot_read(Mesh &m, const double *V, const double *w, int64_t n, int mode, double *out) {
-    const int rows = rows_for(n);
-    k_dot<<<cdiv(n, rows), RED_THREADS, 0, m.stream>>>(V, w, n, rows, m.part.p, m.ticket.p, mode, out, m.h_pinned);
+    k_dot<<<ctas_for(n), RED_THREADS, 0, m.stream>>>(V, w, n, m.part.p, m.ticket.p, mode, out, m.h_pinned);
     BEM_CHECK_LAUNCH();
     BEM_CUDA(cudaStreamSynchronize(m.stream));
     return *const_cast<volatile double *>(m.h_pinned);
 }
 
 double norm2(Mesh &m, const double *w) { return dot_read(m, w, w, m.np, 1, m.red.p); }
+
+// f(NV, MORE) of nvec vectors
+template <int NV = 1, class F>
+static void with_blocks(int nvec, F &&f) {
+    if ((nvec - 1) % VEC_BLOCK + 1 == NV) {
+        if (nvec > VEC_BLOCK) f(std::integral_constant<int, NV>(), std::true_type());
+        else f(std::integral_constant<int, NV>(), std::false_type());
+    } else if constexpr (NV < VEC_BLOCK) {
+        with_blocks<NV + 1>(nvec, f);
+    }
+}
 
 // Solve A x = b (sorted order).  x holds the initial guess on entry; with
 // x_zero the caller knows it to be zero.
@@ -381,7 +441,7 @@ int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bool x_zero
     // an all-zero initial guess skips one product: the residual is b
     const bool told = x_zero;  // red[0] still holds |b|
     if (!x_zero && !conv) x_zero = norm2(m, x) == 0.0;
-    const int rows = rows_for(n), ncta = cdiv(n, rows);
+    const int ncta = ctas_for(n);
     while (!conv && it < m.opt.max_iter && !stagnated) {
         double *V0 = m.V.p;
         const double *r0 = b;
@@ -406,13 +466,21 @@ int gmres_solve(Mesh &m, const double *b, double *x, bool transpose, bool x_zero
             apply(m.V.p + (size_t)j * ld, w);
             ++it;
             // CGS2: two passes of classical Gram-Schmidt
-            k_cgs<<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, j + 1, nullptr, w, n, rows, m.part.p, m.ticket.p, m.hv.p);
-            BEM_CHECK_LAUNCH();
-            k_cgs<<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, j + 1, m.hv.p, w, n, rows, m.part.p, m.ticket.p, m.yv.p);
-            BEM_CHECK_LAUNCH();
-            k_cgs_end<<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, j, m.hv.p, m.yv.p, w, n, rows, m.part.p, m.ticket.p, m.H.p,
-                                                   m1, m.cs.p, m.sn.p, m.gv.p, 1.0 / bnorm, m.red.p, m.h_pinned);
-            BEM_CHECK_LAUNCH();
+            with_blocks(j + 1, [&](auto nv, auto more) {
+                constexpr int NV = decltype(nv)::value;
+                constexpr bool MORE = decltype(more)::value;
+                const int full = j / VEC_BLOCK;
+                k_cgs<NV, false, MORE><<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, full, nullptr, w, n, m.part.p, m.ticket.p,
+                                                                    m.hv.p);
+                BEM_CHECK_LAUNCH();
+                k_cgs<NV, true, MORE><<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, full, m.hv.p, w, n, m.part.p, m.ticket.p,
+                                                                   m.yv.p);
+                BEM_CHECK_LAUNCH();
+                k_cgs_end<NV, MORE><<<ncta, RED_THREADS, 0, s>>>(m.V.p, ld, full, m.hv.p, m.yv.p, w, n, m.part.p,
+                                                                 m.ticket.p, m.H.p, m1, m.cs.p, m.sn.p, m.gv.p,
+                                                                 1.0 / bnorm, m.red.p, m.h_pinned);
+                BEM_CHECK_LAUNCH();
+            });
             k_scale_by<<<nb, 256, 0, s>>>(w, m.red.p + 1, n);
             BEM_CHECK_LAUNCH();
             BEM_CUDA(cudaStreamSynchronize(s));
