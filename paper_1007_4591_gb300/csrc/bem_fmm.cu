@@ -1611,7 +1611,9 @@ static size_t tree_translate_smem(int nc, int cs) {
     const size_t ab = ((size_t)nc * TREE_BM + (size_t)TR_BN_TREE * tree_ldb<T>(cs)) * sizeof(T);
     return std::max(ab, (size_t)TR_BN_TREE * (TREE_BM + 1) * sizeof(T));
 }
-constexpr size_t TREE_SMEM_MAX = 200 * 1024;  // above: the pipelined k_translate
+static_assert(((size_t)(MAXP + 1) * (MAXP + 1) * TREE_BM + TR_BN_TREE * ((MAXP + 1) * (MAXP + 1) + 64)) * sizeof(double) <=
+                  227 * 1024,
+              "an operator block and its input rows fit into a CTA's shared memory at every order");
 
 template <class T, int BN>
 static size_t translate_smem() {
@@ -1948,38 +1950,29 @@ static void clear_expansions(Mesh &m, const Tree &t, T *M, T *L, int cs) {
 // one level of M2M or L2L: the chunks [chunk0, chunk0 + nchunk) of the
 // grouped tree translations
 template <class T>
-static void tree_translate(const T *ops, int nc, int cs, int rblocks, const Tree &t, int chunk0, int nchunk,
-                           const T *in, T *out, cudaStream_t s) {
+static void tree_translate(const T *ops, int nc, int cs, const Tree &t, int chunk0, int nchunk, const T *in, T *out,
+                           cudaStream_t s) {
     if (nchunk == 0) return;
-    dim3 g(nchunk, rblocks);
     const size_t sm = tree_translate_smem<T>(nc, cs);
-    if (sm <= TREE_SMEM_MAX) {
-        dim3 gt(nchunk, cdiv(nc, TREE_BM));
-        auto kern = k_tree_translate<T, TR_BN_TREE, TR_THREADS_TREE, TREE_BM, TREE_RPT>;
-        set_smem<T>(kern, sm);
-        // programmatic dependent launch: the CTAs may start while the previous
-        // kernel of the stream finishes (the kernel waits before it reads its
-        // input or writes its output)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = gt;
-        cfg.blockDim = dim3(TR_THREADS_TREE);
-        cfg.dynamicSmemBytes = sm;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const int ldb = tree_ldb<T>(cs);
-        const int4 *chunks = t.g_chunk.p + chunk0;
-        const int *po = t.g_out.p, *pi = t.g_in.p;
-        BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, ops, nc, cs, ldb, chunks, po, pi, in, out));
-    } else {
-        const size_t trsm_t = translate_smem<T, TR_BN_TREE>();
-        set_smem<T>(k_translate<T, TR_BN_TREE, TR_THREADS_TREE>, trsm_t);
-        k_translate<T, TR_BN_TREE, TR_THREADS_TREE><<<g, TR_THREADS_TREE, trsm_t, s>>>(
-            ops, nc, cs, t.g_chunk.p + chunk0, t.g_out.p, t.g_in.p, in, out);
-    }
+    auto kern = k_tree_translate<T, TR_BN_TREE, TR_THREADS_TREE, TREE_BM, TREE_RPT>;
+    set_smem<T>(kern, sm);
+    // programmatic dependent launch: the CTAs may start while the previous
+    // kernel of the stream finishes (the kernel waits before it reads its
+    // input or writes its output)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nchunk, cdiv(nc, TREE_BM));
+    cfg.blockDim = dim3(TR_THREADS_TREE);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const int ldb = tree_ldb<T>(cs);
+    const int4 *chunks = t.g_chunk.p + chunk0;
+    const int *po = t.g_out.p, *pi = t.g_in.p;
+    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, ops, nc, cs, ldb, chunks, po, pi, in, out));
     BEM_CHECK_LAUNCH();
 }
 
@@ -1993,7 +1986,7 @@ static void tree_sweep(Mesh &m, const T *ops, int nc, int cs, const Tree &t, boo
                        cudaStream_t s) {
     for (int k = 0; k + 3 <= t.L; ++k) {
         const int c = up ? t.L - k : 3 + k;
-        tree_translate<T>(ops, nc, cs, cdiv(nc, TR_BM), t, up ? t.m2m_chunk0[c] : t.l2l_chunk0[c],
+        tree_translate<T>(ops, nc, cs, t, up ? t.m2m_chunk0[c] : t.l2l_chunk0[c],
                           up ? t.m2m_nchunk[c] : t.l2l_nchunk[c], in, out, s);
     }
 }
