@@ -164,7 +164,7 @@ constexpr int P2M_SEG_BATCH = 16;
 
 template <class T>
 __global__ void __launch_bounds__(128)
-k_p2m_seg(TreeView tv, const T *__restrict__ mom, const double *__restrict__ dens, int nc, int cs, T *M) {
+k_p2m_seg(TreeView tv, const T *__restrict__ mom, const double *__restrict__ dens, int nc, int ld, int cs, T *M) {
     // the first upward translation may start now (it waits for this grid's
     // results before it reads them)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -177,13 +177,13 @@ k_p2m_seg(TreeView tv, const T *__restrict__ mom, const double *__restrict__ den
     for (int j = 0; j < NJ; ++j) acc[j] = 0;
     for (int s0 = b; s0 < e; s0 += 128) {
         const int ns = min(128, e - s0);
-        const T *base = mom + (size_t)s0 * cs + threadIdx.x;
+        const T *base = mom + (size_t)s0 * ld + threadIdx.x;
         T v[B];
         auto load = [&](int j, int q0) {
             const bool ok = (int)threadIdx.x + 128 * j < nc;
 #pragma unroll
             for (int u = 0; u < B; ++u)
-                v[u] = (ok && q0 + u < ns) ? __ldg(base + 128 * j + (size_t)(q0 + u) * cs) : (T)0;
+                v[u] = (ok && q0 + u < ns) ? __ldg(base + 128 * j + (size_t)(q0 + u) * ld) : (T)0;
         };
         load(0, 0);
         __syncthreads();
@@ -262,7 +262,7 @@ static bool build_p2m_moments_t(Mesh &m, Tree &t, const typename V4T<T>::t *rec,
     using V4 = typename V4T<T>::t;
     cudaStream_t s = m.stream;
     const int64_t n = m.nqp;
-    const int p = m.opt.p, cs = cell_stride(p);
+    const int p = m.opt.p, ld = moment_stride(p);
     if ((p + 1) * (p + 1) > P2M_SEG_MAXNC || n <= 0 || n >= ((int64_t)1 << 31) || t.nleaf <= 0) return false;
     // the points' (leaf, panel) keys, sorted stably: points already come in
     // leaf order, so each leaf's points end up grouped by panel
@@ -292,7 +292,7 @@ static bool build_p2m_moments_t(Mesh &m, Tree &t, const typename V4T<T>::t *rec,
     BEM_CUDA(cudaStreamSynchronize(s));
     const int nseg = last_pos + last_flag;
     // the moments may take at most half of the free device memory
-    const size_t bytes = (size_t)nseg * cs * sizeof(T);
+    const size_t bytes = (size_t)nseg * ld * sizeof(T);
     size_t fr = 0, tot = 0;
     BEM_CUDA(cudaMemGetInfo(&fr, &tot));
     if (nseg <= 0 || bytes > fr / 2) return false;
@@ -312,14 +312,14 @@ static bool build_p2m_moments_t(Mesh &m, Tree &t, const typename V4T<T>::t *rec,
     rp.alloc(n);
     k_seg_gather<V4><<<cdiv(n, 256), 256, 0, s>>>(rec, idx_s.p, n, rp.p);
     BEM_CHECK_LAUNCH();
-    mom.alloc((size_t)nseg * cs);
+    mom.alloc((size_t)nseg * ld);
     BEM_CUDA(cudaMemsetAsync(mom.p, 0, bytes, s));
     TreeView sv = tv;
     sv.qp_beg = pt_beg.p;
     sv.leaf0 = 0;
     sv.nleaf = nseg;
     const T inv_h = (T)(1.0 / (m.side / (double)(1 << t.L)));
-    p2m_dispatch<T>(sv, nseg, SRC_QUAD, rp.p, nullptr, nullptr, p, cs, inv_h, mom.p, s);
+    p2m_dispatch<T>(sv, nseg, SRC_QUAD, rp.p, nullptr, nullptr, p, ld, inv_h, mom.p, s);
     BEM_CUDA(cudaStreamSynchronize(s));  // the temporaries are released on return
     return true;
 }
@@ -362,7 +362,7 @@ void p2m_leaves(const TreeView &tv, int nleaf, SrcKind sk, const typename V4T<T>
     if (nleaf <= 0) return;
     const T *mom = seg_moments<T>(tv);
     if (sk == SRC_QUAD && tv.seg_beg && mom && tv.seg_p == p) {
-        k_p2m_seg<T><<<nleaf, 128, 0, s>>>(tv, mom, dens, (p + 1) * (p + 1), cs, M);
+        k_p2m_seg<T><<<nleaf, 128, 0, s>>>(tv, mom, dens, (p + 1) * (p + 1), moment_stride(p), cs, M);
         BEM_CHECK_LAUNCH();
         return;
     }
