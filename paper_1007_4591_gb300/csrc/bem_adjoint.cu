@@ -129,6 +129,7 @@ static void direct_adjoint(Mesh &m, AdjSrc sk, AdjTgt tk, const double *dens, do
     // splits of at least 4,096 sources (FP64) or 512 (FP32: a CTA is four warps,
     // and a thousand charges give few blocks of targets)
     int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, f32 ? 512 : 4096), std::max(1, (f32 ? 4 * 8 * 152 : 1216) / tblocks)));
+    if (f32) nsplit = std::min(nsplit, std::max({splits_limit(m, ntgt * no), std::min(cdiv(nsrc, 4096), 1216 / tblocks), 1}));
     nsplit = std::min(nsplit, 65535);
     int64_t chunk = (nsrc + nsplit - 1) / nsplit;
     chunk = ((chunk + ADJ_THREADS - 1) / ADJ_THREADS) * ADJ_THREADS;
@@ -145,6 +146,7 @@ static void direct_adjoint(Mesh &m, AdjSrc sk, AdjTgt tk, const double *dens, do
     d.qpanel = sk == AS_QUAD ? m.qp_panel.p : nullptr;
     d.dens = gq ? m.lamq.p : (sk == AS_CHARGE ? nullptr : dens);
     d.tpos = (tk == AT_CHG_GRAD) ? m.chgg64.p : m.qpg64.p;
+    d.to_quad_values = out == quad_values(m);
     const size_t need = (size_t)nsplit * ntgt * no;
     if (f32) {
         if (m.dpart_f.n < need) m.dpart_f.alloc(need);
@@ -201,10 +203,10 @@ __global__ void k_gradients(const double *cs4, const double *bl4, const double *
 void build_qp_of_panel(Mesh &m);
 
 AdjointVectors adjoint_vectors(Mesh &m) {
-    const size_t nc = (size_t)m.nc, np = (size_t)m.np, need = 12 * nc + 2 * np + (size_t)m.nqp;
+    const size_t nc = (size_t)m.nc, np = (size_t)m.np, need = 12 * nc + np;
     if (m.adj.n < need) m.adj.alloc(need);
     double *p = m.adj.p;
-    return AdjointVectors{p, p + 4 * nc, p + 8 * nc, p + 9 * nc, p + 12 * nc, p + 12 * nc + np, p + 12 * nc + 2 * np};
+    return AdjointVectors{p, p + 4 * nc, p + 8 * nc, p + 9 * nc, p + 12 * nc};
 }
 
 void adjoint_gradients(Mesh &m, double grad_out, double *dq_s, double *dx_s) {
@@ -212,7 +214,7 @@ void adjoint_gradients(Mesh &m, double grad_out, double *dq_s, double *dx_s) {
     build_qp_of_panel(m);
     const int64_t np = m.np, nc = m.nc;
     const AdjointVectors v = adjoint_vectors(m);
-    double *cs4 = v.cs4, *bl4 = v.bl4, *lam = v.lam, *rhs = v.rhs, *psi = v.psi;
+    double *cs4 = v.cs4, *bl4 = v.bl4, *lam = v.lam, *rhs = rhs_vector(m), *psi = quad_values(m);
     // C sigma and its gradient at the charges
     direct_adjoint(m, AS_QUAD, AT_CHG_GRAD, m.sigma_s.p, cs4);
     charge_near_phi(m, m.sigma_s.p, cs4, 4, 4);

@@ -139,7 +139,7 @@ size_t Mesh::bytes() const {
     b += lamq.bytes() + pan64.bytes() + cn_off.bytes() + cn_col.bytes() + cn_val.bytes() + cnT_off.bytes() + cnT_row.bytes() +
          cnT_val.bytes();
     b += ctq.bytes() + str32.bytes() + str64.bytes() + near64.bytes() + dpart_f.bytes() +
-         dpart_d.bytes() + dsrc.bytes();
+         dpart_d.bytes();
     b += xs.bytes() + ys.bytes() + zs.bytes() + far_f.bytes() + near_f.bytes() + far_d.bytes() +
          near_d.bytes() + io_a.bytes() + io_b.bytes() + red.bytes();
     b += dev_err.bytes();
@@ -171,7 +171,7 @@ static void alloc_work(Mesh &m) {
     }
     // near-field source pairs: each leaf padded to an even count
     const size_t nsrc = (size_t)std::max<int64_t>(m.nqp, m.nc) + (size_t)std::max(m.tp.nleaf, m.tc.nleaf) + 4;
-    if (m.opt.precision == BEM_MIXED) ensure(m.str32, nsrc);
+    if (m.opt.precision == BEM_MIXED) ensure(m.str32, std::max(nsrc, direct_space(m)));
     else ensure(m.str64, nsrc);
     ensure(m.near64, (size_t)m.np);
     const size_t nv = (size_t)std::max<int64_t>(m.np, m.nc);
@@ -412,12 +412,6 @@ static void rhs_sorted(Mesh &m, double *b_s) {
     }
     charge_pass(m, SRC_CHARGE, m.opt.galerkin ? TGT_QUAD_DN : TGT_CEN_DN, nullptr, m.zs.p);
     axpby(m, -m.ehat, m.zs.p, 0.0, m.zs.p, b_s, m.np);
-}
-
-// the solve's right-hand side, kept with the mesh
-static double *rhs_vector(Mesh &m) {
-    if (m.bvec.n < (size_t)m.np) m.bvec.alloc(m.np);
-    return m.bvec.p;
 }
 
 int bem_rhs(bem_mesh *m, double *b) {

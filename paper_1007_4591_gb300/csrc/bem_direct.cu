@@ -266,20 +266,36 @@ k_direct_pk(int64_t ntgt, int64_t nsrc, int64_t chunk, int64_t seg0, int64_t seg
         }
 }
 
-// Sources are packed and summed a segment at a time (at most 2^20 sources, 32
-// or 48 MB of records; smaller where the device has no room).
+double *quad_values(Mesh &m) {
+    return reinterpret_cast<double *>(m.opt.precision == BEM_MIXED ? (void *)m.str32.p : (void *)m.str64.p);
+}
+
+size_t direct_space(const Mesh &m) { return (size_t)(m.nqp + 1) / 2 + DREC_DIPOLE * DIRECT_TILE; }
+
+// The records of a call live in memory that only products and GMRES use
+// otherwise: the near field's strength records (16 bytes a quadrature point,
+// less the values at the points when the call writes those) or, once a solve
+// has run, its basis (31 vectors: room for every point's two records).
+static void record_space(Mesh &m, bool values, float4 *&rec, size_t &n) {
+    const size_t keep = values ? (size_t)(m.nqp + 1) / 2 : 0;
+    rec = m.str32.p + keep;
+    n = m.str32.n - keep;
+    if (m.V.n / 2 > n) {
+        rec = reinterpret_cast<float4 *>(m.V.p);
+        n = m.V.n / 2;
+    }
+}
+
+// Sources are packed and summed a segment at a time: as many whole tiles as
+// there is room for (the tiles' sums do not depend on it).
 void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, float *part) {
     cudaStream_t s = m.stream;
     const int rs = d.dipole ? DREC_DIPOLE : DREC_MONO;
-    int64_t seg = std::min<int64_t>((d.nsrc + DIRECT_TILE - 1) / DIRECT_TILE * DIRECT_TILE, (int64_t)1 << 20);
-    while (m.dsrc.n < (size_t)(seg * rs)) {
-        try {
-            m.dsrc.alloc((size_t)(seg * rs));
-        } catch (const Error &e) {
-            if (e.code != BEM_ENOMEM || seg <= 64 * DIRECT_TILE) throw;
-            seg /= 2;
-        }
-    }
+    float4 *rec;
+    size_t room;
+    record_space(m, d.to_quad_values, rec, room);
+    const int64_t seg = (int64_t)(room / rs / DIRECT_TILE * DIRECT_TILE);
+    if (seg == 0) throw Error(BEM_ECUDA, "direct sums: no room for a tile of records");
     const double ox = m.root_min[0] + 0.5 * m.side, oy = m.root_min[1] + 0.5 * m.side,
                  oz = m.root_min[2] + 0.5 * m.side;
     const size_t sm = (size_t)2 * DIRECT_TILE * rs * sizeof(float4);
@@ -288,12 +304,12 @@ void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, flo
         const double *sw = d.sw ? d.sw + s0 : nullptr, *dens = d.dens && !d.qpanel ? d.dens + s0 : d.dens;
         auto pack = d.dipole ? k_direct_pack<true> : k_direct_pack<false>;
         pack<<<cdiv(n, 256), 256, 0, s>>>(n, d.spos + 3 * s0, sw, d.snrm ? d.snrm + 3 * s0 : nullptr,
-                                          d.qpanel ? d.qpanel + s0 : nullptr, dens, ox, oy, oz, m.dsrc.p);
+                                          d.qpanel ? d.qpanel + s0 : nullptr, dens, ox, oy, oz, rec);
         BEM_CHECK_LAUNCH();
         const int y0 = (int)(s0 / chunk), y1 = std::min(nsplit, (int)((s1 - 1) / chunk) + 1);
         auto go = [&](auto kern) {
             kern<<<dim3(cdiv(d.ntgt, DPK_TARGETS), y1 - y0), DPK_THREADS, sm, s>>>(
-                d.ntgt, d.nsrc, chunk, s0, s1, y0, d.tpos, d.tnrm, m.dsrc.p, ox, oy, oz, part);
+                d.ntgt, d.nsrc, chunk, s0, s1, y0, d.tpos, d.tnrm, rec, ox, oy, oz, part);
             BEM_CHECK_LAUNCH();
         };
         if (d.dipole && d.kind == DO_PHI_GRAD) go(k_direct_pk<true, DO_PHI_GRAD, true>);
@@ -377,6 +393,8 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
     constexpr bool F32 = std::is_same<T, float>::value;
     const int ctas = F32 && sk == SRC_QUAD ? 4 * 10 * 152 : 2432;
     int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, 512), std::max(1, ctas / tblocks)));
+    if (F32 && sk == SRC_QUAD)
+        nsplit = std::min(nsplit, std::max({splits_limit(m, ntgt), 2432 / tblocks, 1}));
     nsplit = std::min(nsplit, 65535);
     int64_t chunk = (nsrc + nsplit - 1) / nsplit;
     chunk = ((chunk + DIRECT_THREADS - 1) / DIRECT_THREADS) * DIRECT_THREADS;
@@ -384,8 +402,7 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
     // added in order by the reduction (the sums a CTA per split gives, in
     // shorter CTAs: 81,920 targets, 2,000 charges are 1.2 waves of splits)
     int group = 1;
-    // (while the parts stay below 64 MB)
-    if (F32 && sk == SRC_CHARGE && (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= 1.6e7) {
+    if (F32 && sk == SRC_CHARGE && (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= parts_limit(m)) {
         group = (int)(chunk / DIRECT_TILE);
         chunk = DIRECT_TILE;
     }
@@ -412,6 +429,7 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
         d.qpanel = qpanel;
         d.tpos = tpos;
         d.tnrm = tnrm;
+        d.to_quad_values = out == quad_values(m);
         direct_partials(m, d, chunk, nsplit, part.p);
     } else {
         dim3 grid(tblocks, nsplit);
@@ -459,7 +477,7 @@ void build_ctq(Mesh &m) {
     m.ctq_ok = false;
     if (m.nc == 0 || !charge_direct(m)) return;
     if (m.ctq.n < (size_t)m.np) m.ctq.alloc(m.np);
-    double *psi = adjoint_vectors(m).psi;
+    double *psi = quad_values(m);
     direct_pass(m, SRC_CHARGE, TGT_QUAD_PHI, nullptr, psi);
     panel_wsum(m, psi, m.ctq.p);
     charge_near_ct(m, m.q64.p, m.ctq.p);

@@ -331,12 +331,11 @@ struct Mesh {
     DArray<double> red;                // reduction scratch
     DArray<float> dpart_f;             // direct-sum partials (mixed)
     DArray<double> dpart_d;            // direct-sum partials (fp64)
-    DArray<float4> dsrc;               // direct-sum source records of one segment (mixed)
     double *h_pinned = nullptr;        // small pinned host buffer
 
     // GMRES workspace
     DArray<double> V, H, gv, cs, sn, yv, hv, part;
-    DArray<double> bvec;               // the solve's right-hand side
+    DArray<double> bvec;               // right-hand side of the system at hand
     DArray<unsigned> ticket;           // arrivals of a reduction's CTAs
     // last solve (for the adjoint)
     DArray<double> sigma_s;
@@ -446,10 +445,10 @@ void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *ou
 bool charge_direct(const Mesh &m);
 void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out);
 void build_ctq(Mesh &m);
-// the adjoint gradients' vectors, kept with the mesh: (phi, grad) of C sigma and
-// of B^T lam, the gradients, lam, C^T q, the charges' potential at the points
+// the adjoint gradients' vectors, kept with the mesh from its first gradient on:
+// (phi, grad) of C sigma and of B^T lam, the gradients, lam
 struct AdjointVectors {
-    double *cs4, *bl4, *gq, *gx, *lam, *rhs, *psi;
+    double *cs4, *bl4, *gq, *gx, *lam;
 };
 AdjointVectors adjoint_vectors(Mesh &m);
 // All-pairs sums in FP32 with split coordinates (bem_direct.cu), shared by the
@@ -458,12 +457,23 @@ enum DirectOut { DO_DN, DO_PHI, DO_PHI_GRAD };  // normal field, potential, pote
 struct DirectSum {
     bool dipole = false;           // moments dens[k] nrm[k] instead of strengths
     bool skip_coincident = false;  // a pair at distance 0 adds nothing
+    bool to_quad_values = false;   // the call's output is quad_values
     DirectOut kind = DO_PHI;
     int64_t nsrc = 0, ntgt = 0;
     const double *spos = nullptr, *sw = nullptr, *snrm = nullptr, *dens = nullptr;
     const int *qpanel = nullptr;   // strengths sw[k] dens[qpanel[k]] (else dens[k], or sw[k] without dens)
     const double *tpos = nullptr, *tnrm = nullptr;
 };
+// one value per quadrature point, in memory that the next product overwrites
+double *quad_values(Mesh &m);
+// 16-byte values that the near field's strength records need to hold at least,
+// for quad_values and a tile of source records beside them
+size_t direct_space(const Mesh &m);
+// FP32 partial sums that a direct sum may keep: 64 a panel (256 bytes, of some
+// 2,500 a mesh holds for it), where a few waves of CTAs need fewer anyway
+inline double parts_limit(const Mesh &m) { return 64.0 * (double)m.np; }
+// the splits of a sum of `values` numbers that stay below it
+inline int splits_limit(const Mesh &m, int64_t values) { return (int)std::min(65535.0, parts_limit(m) / (double)values); }
 // part[split][target] (x 4 with the gradient), split s over the sources [s chunk, (s + 1) chunk)
 void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, float *part);
 // out[n][no] = 1/(4 pi) x the sum over the splits of part[split][n][no], each
@@ -475,6 +485,7 @@ void panel_wsum(Mesh &m, const double *v, double *out);
 double energy_from_ctq(Mesh &m, const double *sig_s);
 
 // solver pieces (bem_solver.cu)
+double *rhs_vector(Mesh &m);
 void matvec_sorted(Mesh &m, const double *xs, double *ys);
 void matvec_t_sorted(Mesh &m, const double *xs, double *ys);
 void exclusive_scan_int(const int *in, int *out, int n, cudaStream_t s);

@@ -396,6 +396,12 @@ static double dot_read(Mesh &m, const double *V, const double *w, int64_t n, int
 
 double norm2(Mesh &m, const double *w) { return dot_read(m, w, w, m.np, 1, m.red.p); }
 
+// the right-hand side of the system at hand
+double *rhs_vector(Mesh &m) {
+    if (m.bvec.n < (size_t)m.np) m.bvec.alloc(m.np);
+    return m.bvec.p;
+}
+
 // f(NV, MORE) of nvec vectors
 template <int NV = 1, class F>
 static void with_blocks(int nvec, F &&f) {
