@@ -2102,16 +2102,21 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
     // 0.272 in two parts, the second released once M2L holds the SMs.  (While
     // the tree kernels took 63 KB and 256 threads a CTA they waited for three
     // near-field CTAs of one SM to end at once: 0.279 ms forked at the start.)
-    if (conc) {
+    // The complex M2L (m2l_mode 2) reads whole rows of scattered cells for
+    // milliseconds and loses more beside the near field than the overlap gains:
+    // there it forks after the upward sweep (40,500 panels in FP64 10.7 ms, 12.1
+    // forked at the start; mixed 0.655 and 0.67).
+    const bool dense = m.opt.m2l_mode != BEM_M2L_DIRECT;
+    auto fork_near = [&]() {
         BEM_CUDA(cudaEventRecord(m.ev_fork, s));
         BEM_CUDA(cudaStreamWaitEvent(m.stream2, m.ev_fork, 0));
         launch_near(m.stream2);
         BEM_CUDA(cudaEventRecord(m.ev_join, m.stream2));
-    }
+    };
+    if (conc && (dense || !far)) fork_near();
     if (far) {
         T *M = B::M(m), *L = B::L(m);
         const int cs = cell_stride(p);
-        const bool dense = m.opt.m2l_mode != BEM_M2L_DIRECT;
         const int rblocks = cdiv(nc, TR_BM);
         const size_t trsm = translate_smem<T, TR_BN_M2L>();
         if (dense) set_smem<T>(k_translate<T, TR_BN_M2L, TR_THREADS>, trsm);
@@ -2132,6 +2137,7 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
             }
         }
         ev_rec(m, timed, 2);
+        if (conc && !dense) fork_near();
         // M2L: every cell at levels 2..L
         if (dense) {
             const int kind = !t.has_chg ? Tree::M2L_ALL : (sk == SRC_CHARGE ? Tree::M2L_CHG_TO_PANEL : Tree::M2L_PANEL_TO_CHG);
