@@ -155,7 +155,7 @@ static void ensure(DArray<T> &d, size_t n) {
 
 // Work buffers (grow-only: a captured graph keeps pointing at them).
 static void alloc_work(Mesh &m) {
-    const size_t nc = (size_t)cell_stride(m.opt.p);
+    const size_t nc = (size_t)cell_stride(m);
     const size_t ncell = (size_t)std::max(m.tp.ncell, m.tc.ncell);
     const size_t nt = (size_t)std::max<int64_t>(std::max<int64_t>(m.np, m.nc), m.nqp);
     if (m.opt.precision == BEM_MIXED) {

@@ -1304,7 +1304,7 @@ static std::map<TabKey, std::weak_ptr<Tables>> g_tab_cache;
 template <class T>
 static void fill_tables(int p, int ws, DArray<T> &R, DArray<T> &I, DArray<T> &om2l, DArray<T> &om2m, DArray<T> &ol2l,
                         DArray<float> *tc, cudaStream_t s) {
-    const int nc = (p + 1) * (p + 1), ld = cell_stride(p), ncls = m2l_classes(ws);
+    const int nc = (p + 1) * (p + 1), ld = row_stride(p), ncls = m2l_classes(ws);
     const size_t nr = (size_t)(p + 1) * (2 * p + 1), ni = (size_t)(2 * p + 1) * (4 * p + 1);
     R.alloc(8 * nr * 2);
     I.alloc(ncls * ni * 2);
@@ -1388,12 +1388,12 @@ __device__ __forceinline__ void cp_async_elt(T *dst, const T *src, bool ok) {
 // out[p_out[j]] += Op[class] x in[p_in[j]] for the pairs of one chunk (one
 // operator class): a [BM x nc] x [nc x BN] product whose K loop is staged
 // through TR_NS shared-memory buffers by cp.async (the operator rows, padded
-// to the cell stride, in 16-byte copies), so every tile's loads are in flight
+// to row_stride, in 16-byte copies), so every tile's loads are in flight
 // together.  NTH threads; each owns 8 consecutive output rows (two or four
 // 16-byte shared loads per k) and BN x 16 / NTH pair columns.
 template <class T, int BN, int NTH>
 __global__ void __launch_bounds__(NTH)
-k_translate(const T *__restrict__ ops, int nc, int cs, const int4 *__restrict__ chunks,
+k_translate(const T *__restrict__ ops, int nc, int ld, int cs, const int4 *__restrict__ chunks,
             const int *__restrict__ p_out, const int *__restrict__ p_in, const T *__restrict__ in,
             T *__restrict__ out) {
     constexpr int BK = TrBK<T>::v;
@@ -1408,7 +1408,7 @@ k_translate(const T *__restrict__ ops, int nc, int cs, const int4 *__restrict__ 
     T *Cs = sm;                             // [BN][BM+1] (epilogue)
     __shared__ int s_in[BN], s_out[BN];
     const int4 ch = chunks[blockIdx.x];
-    const T *Tt = ops + (size_t)ch.x * nc * cs;
+    const T *Tt = ops + (size_t)ch.x * nc * ld;
     const int rb = blockIdx.y * TR_BM;
     const int tid = threadIdx.x, ty = tid / NTX, tx = tid - ty * NTX;
     if (tid < BN) {
@@ -1428,8 +1428,8 @@ k_translate(const T *__restrict__ ops, int nc, int cs, const int4 *__restrict__ 
         const int k0 = kt * BK;
         for (int e = tid; e < BK * TR_BM / VEC; e += NTH) {
             const int k = e / (TR_BM / VEC), r = (e - k * (TR_BM / VEC)) * VEC;
-            const bool ok = k0 + k < nc && rb + r < cs;  // cs % VEC == 0: a copy never crosses a row
-            cp_async_16(As + k * TR_BM + r, ok ? Tt + (size_t)(k0 + k) * cs + rb + r : Tt, ok);
+            const bool ok = k0 + k < nc && rb + r < ld;  // ld % VEC == 0: a copy never crosses a row
+            cp_async_16(As + k * TR_BM + r, ok ? Tt + (size_t)(k0 + k) * ld + rb + r : Tt, ok);
         }
         for (int e = tid; e < BK * BN; e += NTH) {
             const int k = e / BN, j = e - k * BN;
@@ -1499,7 +1499,7 @@ k_translate(const T *__restrict__ ops, int nc, int cs, const int4 *__restrict__ 
 // strided by NTX; input rows padded to 4 mod 32 words: at most 2-way bank
 // conflicts) and the results leave as coalesced atomic adds.
 template <class T, int BN, int NTH, int BM, int RPT>
-__device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, int nc, int cs, int ldb, int4 ch,
+__device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, int nc, int ld, int cs, int ldb, int4 ch,
                                                      int rb, const int *__restrict__ p_out,
                                                      const int *__restrict__ p_in, const T *__restrict__ in,
                                                      T *__restrict__ out, unsigned char *smraw, int *s_in,
@@ -1513,7 +1513,7 @@ __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, 
     T *As = reinterpret_cast<T *>(smraw);  // [nc][TR_BM]
     T *Bs = As + (size_t)nc * TR_BM;       // [BN][ldb]
     T *Cs = As;                            // [BN][TR_BM + 1] (epilogue)
-    const T *Tt = ops + (size_t)ch.x * nc * cs;
+    const T *Tt = ops + (size_t)ch.x * nc * ld;
     // a warp covers 8 pair columns and 4 row groups: its input-row loads hit 8
     // different banks and its operator loads one 128-byte span
     static_assert(NTX % 8 == 0, "tree translate thread map");
@@ -1528,14 +1528,14 @@ __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, 
     __syncthreads();
     for (int e = tid; e < nc * (TR_BM / VEC); e += NTH) {
         const int k = e / (TR_BM / VEC), r = (e - k * (TR_BM / VEC)) * VEC;
-        const bool ok = rb + r < cs;  // cs % VEC == 0: a copy never crosses a row
-        cp_async_16(As + (size_t)k * TR_BM + r, ok ? Tt + (size_t)k * cs + rb + r : Tt, ok);
+        const bool ok = rb + r < ld;  // ld % VEC == 0: a copy never crosses a row
+        cp_async_16(As + (size_t)k * TR_BM + r, ok ? Tt + (size_t)k * ld + rb + r : Tt, ok);
     }
     // everything the previous kernels of the stream wrote (this level's input
     // expansions, the cleared outputs) is complete and visible after this
     // wait; nothing above reads or writes it
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int cv = cs / VEC;
+    const int cv = ld / VEC;  // the coefficients of a row
     for (int e = tid; e < BN * cv; e += NTH) {
         const int j = e / cv, q = (e - j * cv) * VEC;
         const int src = s_in[j];
@@ -1590,25 +1590,28 @@ __device__ __forceinline__ void tree_translate_block(const T *__restrict__ ops, 
 
 template <class T, int BN, int NTH, int BM, int RPT>
 __global__ void __launch_bounds__(NTH)
-k_tree_translate(const T *__restrict__ ops, int nc, int cs, int ldb, const int4 *__restrict__ chunks,
+k_tree_translate(const T *__restrict__ ops, int nc, int ld, int cs, int ldb, const int4 *__restrict__ chunks,
                  const int *__restrict__ p_out, const int *__restrict__ p_in, const T *__restrict__ in,
                  T *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_in[BN], s_out[BN];
-    tree_translate_block<T, BN, NTH, BM, RPT>(ops, nc, cs, ldb, chunks[blockIdx.x], blockIdx.y * BM, p_out, p_in, in, out,
-                                         smraw, s_in, s_out);
+    tree_translate_block<T, BN, NTH, BM, RPT>(ops, nc, ld, cs, ldb, chunks[blockIdx.x], blockIdx.y * BM, p_out, p_in, in,
+                                              out, smraw, s_in, s_out);
 }
 
-// input-row pitch of k_tree_translate (4 mod 32 words) and its shared memory
+// input-row pitch of k_tree_translate, the least that is 4 mod 32 words (at
+// p = 16, 292 values, three CTAs fit into an SM instead of two: M2M 36 -> 29 us,
+// 40,500 panels), and its shared memory
 template <class T>
-static int tree_ldb(int cs) {
-    return (int)(((cs * sizeof(T) + 127) / 128 * 128 + 16) / sizeof(T));
+static int tree_ldb(int ld) {
+    const int w = (int)(sizeof(T) / 4);
+    return ld + (36 - ld * w % 32) % 32 / w;
 }
 constexpr int TREE_BM = 32;  // operator rows per CTA (four CTAs per chunk at p = 10)
 constexpr int TREE_RPT = 4;  // rows per thread
 template <class T>
-static size_t tree_translate_smem(int nc, int cs) {
-    const size_t ab = ((size_t)nc * TREE_BM + (size_t)TR_BN_TREE * tree_ldb<T>(cs)) * sizeof(T);
+static size_t tree_translate_smem(int nc, int ld) {
+    const size_t ab = ((size_t)nc * TREE_BM + (size_t)TR_BN_TREE * tree_ldb<T>(ld)) * sizeof(T);
     return std::max(ab, (size_t)TR_BN_TREE * (TREE_BM + 1) * sizeof(T));
 }
 static_assert(((size_t)(MAXP + 1) * (MAXP + 1) * TREE_BM + TR_BN_TREE * ((MAXP + 1) * (MAXP + 1) + 64)) * sizeof(double) <=
@@ -1950,10 +1953,10 @@ static void clear_expansions(Mesh &m, const Tree &t, T *M, T *L, int cs) {
 // one level of M2M or L2L: the chunks [chunk0, chunk0 + nchunk) of the
 // grouped tree translations
 template <class T>
-static void tree_translate(const T *ops, int nc, int cs, const Tree &t, int chunk0, int nchunk, const T *in, T *out,
+static void tree_translate(const T *ops, int nc, int ld, int cs, const Tree &t, int chunk0, int nchunk, const T *in, T *out,
                            cudaStream_t s) {
     if (nchunk == 0) return;
-    const size_t sm = tree_translate_smem<T>(nc, cs);
+    const size_t sm = tree_translate_smem<T>(nc, ld);
     auto kern = k_tree_translate<T, TR_BN_TREE, TR_THREADS_TREE, TREE_BM, TREE_RPT>;
     set_smem<T>(kern, sm);
     // programmatic dependent launch: the CTAs may start while the previous
@@ -1969,10 +1972,10 @@ static void tree_translate(const T *ops, int nc, int cs, const Tree &t, int chun
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const int ldb = tree_ldb<T>(cs);
+    const int ldb = tree_ldb<T>(ld);
     const int4 *chunks = t.g_chunk.p + chunk0;
     const int *po = t.g_out.p, *pi = t.g_in.p;
-    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, ops, nc, cs, ldb, chunks, po, pi, in, out));
+    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, ops, nc, ld, cs, ldb, chunks, po, pi, in, out));
     BEM_CHECK_LAUNCH();
 }
 
@@ -1986,7 +1989,7 @@ static void tree_sweep(Mesh &m, const T *ops, int nc, int cs, const Tree &t, boo
                        cudaStream_t s) {
     for (int k = 0; k + 3 <= t.L; ++k) {
         const int c = up ? t.L - k : 3 + k;
-        tree_translate<T>(ops, nc, cs, t, up ? t.m2m_chunk0[c] : t.l2l_chunk0[c],
+        tree_translate<T>(ops, nc, row_stride(m.opt.p), cs, t, up ? t.m2m_chunk0[c] : t.l2l_chunk0[c],
                           up ? t.m2m_nchunk[c] : t.l2l_nchunk[c], in, out, s);
     }
 }
@@ -2116,7 +2119,7 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
     if (conc && (dense || !far)) fork_near();
     if (far) {
         T *M = B::M(m), *L = B::L(m);
-        const int cs = cell_stride(p);
+        const int cs = cell_stride(m);
         const int rblocks = cdiv(nc, TR_BM);
         const size_t trsm = translate_smem<T, TR_BN_M2L>();
         if (dense) set_smem<T>(k_translate<T, TR_BN_M2L, TR_THREADS>, trsm);
@@ -2483,7 +2486,7 @@ static void m2l_dense(Mesh &m, const Tree &t, const Tree::M2LPairs &g, const T *
     }
     if (g.nchunk == 0) return;
     k_translate<T, TR_BN_M2L, TR_THREADS><<<dim3(g.nchunk, rblocks), TR_THREADS, trsm, m.stream>>>(
-        Oop, nc, cs, g.chunk.p, g.out.p, g.in.p, M, L);
+        Oop, nc, row_stride(m.opt.p), cs, g.chunk.p, g.out.p, g.in.p, M, L);
     BEM_CHECK_LAUNCH();
 }
 
@@ -2512,7 +2515,7 @@ static void run_pass_t(Mesh &m, const double *lam, double *out) {
     const Tables &tb = tables_for(m, t);
     const int p = m.opt.p;
     const int nc = (p + 1) * (p + 1);
-    const int cs = cell_stride(p);
+    const int cs = cell_stride(m);
     const double h = m.side / (double)(1 << t.L);
     const T inv_h = (T)(1.0 / h);
     const bool far = !(m.opt.flags & BEM_FLAG_NO_FAR) && t.L >= 2;

@@ -179,8 +179,8 @@ struct Tree {
     // M_leaf = sum over the leaf's segments of sigma(panel) x moment.
     DArray<int> p2m_seg_beg;      // [nleaf+1] the segments of each leaf (CSR)
     DArray<int> p2m_seg_panel;    // [nseg] panel of each segment
-    DArray<float> p2m_seg_f;      // [nseg x moment stride] moments (mixed precision)
-    DArray<double> p2m_seg_d;     // [nseg x moment stride] moments (FP64)
+    DArray<float> p2m_seg_f;      // [nseg x row stride] moments (mixed precision)
+    DArray<double> p2m_seg_d;     // [nseg x row stride] moments (FP64)
     int p2m_seg_p = -1;           // expansion order of the moments (-1: none built)
     std::vector<int> m2m_chunk0, m2m_nchunk, l2l_chunk0, l2l_nchunk; // indexed by child level
     size_t bytes() const;
@@ -219,7 +219,7 @@ struct Mesh;
 //   If:   irregular harmonics I_n^m (n <= 2p) of the 343 offset classes;
 //   Om2l, Om2m, Ol2l: the translations as real (p+1)^2 x (p+1)^2 matrices
 //         in the compact real layout, stored column-major ([in][out]) with
-//         each [in] row padded with zeros to the cell stride.
+//         each [in] row padded with zeros to row_stride.
 struct Tables {
     int p = 0;
     int ws = 1;                   // the M2L operators cover the offset classes of this separation
@@ -349,17 +349,9 @@ struct Mesh {
 
 // --------------------------------------------------------------- helpers
 inline int ncoef(int p) { return (p + 1) * (p + 1); }
-// the tensor-core kernel's M2L operators are TC_TABLE_DIM^2 values
-constexpr int TC_TABLE_DIM = 128;
-// stride of the panel moments' rows: (p+1)^2 rounded up to 4 values
-inline int moment_stride(int p) { return (ncoef(p) + 3) & ~3; }
-// stride of the expansion arrays' and the operators' rows: 4 values again, or
-// 32 (rows on whole 128-byte lines) at the orders the tensor-core M2L serves:
-// its copies and reductions want lines, the sweeps gain 2 % from them (40,500
-// panels, p = 10: 0.1995 -> 0.1965 ms).  At p = 12, where the SIMT kernel
-// carries the M2L, rows of 192 instead of 172 values took 1.20 against 1.04 ms
-// (81,920 panels).
-inline int cell_stride(int p) { return ncoef(p) <= TC_TABLE_DIM ? (ncoef(p) + 31) & ~31 : moment_stride(p); }
+// stride of the operators' and the panel moments' rows: (p+1)^2 rounded up to
+// 4 values (16-byte copies)
+inline int row_stride(int p) { return (ncoef(p) + 3) & ~3; }
 inline int cdiv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // geometry + trees (bem_tree.cu)
@@ -413,12 +405,19 @@ bool tc_m2l_available(const Mesh &m);
 // class (zero-padded), [in / 4][out][in % 4], so that the kernel writes output
 // coefficient `out` into tensor-memory lane `out` and the 32 lanes of a warp
 // read 4 consecutive input coefficients each from 512 contiguous bytes
+constexpr int TC_TABLE_DIM = 128;
 __host__ __device__ inline int tc_table_index(int in, int out) {
     return ((in >> 2) * TC_TABLE_DIM + out) * 4 + (in & 3);
 }
 void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cudaStream_t s);
 void m2l_tc(Mesh &m, const Tree &t, const Tree::M2LPairs &g, const float *M, float *L, bool timed = false);
 bool use_tc_m2l(const Mesh &m);
+// stride of the expansions' rows: row_stride, or 32 values (rows on whole
+// 128-byte lines) where the tensor-core M2L copies and reduces them (40,500
+// panels, p = 10: the product 200 -> 197 us).  The SIMT M2L's atomics meet on
+// rows of 128 values: 348 instead of 288 us (81,920 panels, p = 10), and at
+// p = 12 rows of 192 instead of 172 took the product from 1.04 to 1.20 ms.
+inline int cell_stride(const Mesh &m) { return use_tc_m2l(m) ? (ncoef(m.opt.p) + 31) & ~31 : row_stride(m.opt.p); }
 void compute_bbox(const double *d, int64_t n, int stride, double *lo, double *hi, cudaStream_t s);
 
 // fast multipole passes (bem_fmm.cu).  `dens` is indexed in sorted panel

@@ -264,7 +264,7 @@ static bool build_p2m_moments_t(Mesh &m, Tree &t, const typename V4T<T>::t *rec,
     using V4 = typename V4T<T>::t;
     cudaStream_t s = m.stream;
     const int64_t n = m.nqp;
-    const int p = m.opt.p, ld = moment_stride(p);
+    const int p = m.opt.p, ld = row_stride(p);
     if ((p + 1) * (p + 1) > P2M_SEG_MAXNC || n <= 0 || n >= ((int64_t)1 << 31) || t.nleaf <= 0) return false;
     // the points' (leaf, panel) keys, sorted stably: points already come in
     // leaf order, so each leaf's points end up grouped by panel
@@ -364,7 +364,7 @@ void p2m_leaves(const TreeView &tv, int nleaf, SrcKind sk, const typename V4T<T>
     if (nleaf <= 0) return;
     const T *mom = seg_moments<T>(tv);
     if (sk == SRC_QUAD && tv.seg_beg && mom && tv.seg_p == p) {
-        k_p2m_seg<T><<<nleaf, 128, 0, s>>>(tv, mom, dens, (p + 1) * (p + 1), moment_stride(p), cs, M);
+        k_p2m_seg<T><<<nleaf, 128, 0, s>>>(tv, mom, dens, (p + 1) * (p + 1), row_stride(p), cs, M);
         BEM_CHECK_LAUNCH();
         return;
     }

@@ -548,7 +548,7 @@ void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cuda
 void m2l_tc(Mesh &m, const Tree &t, const Tree::M2LPairs &g, const float *M, float *L, bool timed) {
     const Tables &tb = tables_for(m, t);
     const int nc = (m.opt.p + 1) * (m.opt.p + 1);
-    const int cs = cell_stride(m.opt.p);
+    const int cs = cell_stride(m);
     if (g.nsuper == 0) return;
     const bool tk = timed && m.tm.on && m.tm.kev[0];
     auto kev = [&](int k) {
