@@ -1636,37 +1636,66 @@ __global__ void k_class_count(const int *key, int64_t n, int *cnt) {
     if (i < n) atomicAdd(cnt + key[i], 1);
 }
 
-// grouped pair d is list entry e = perm[d]
-__global__ void k_gather_pairs(const int *perm, const int *po, const int *pi, int64_t n, int *g_out, int *g_in) {
+// grouped pair d is entry e = perm[d]; the first n0 go to one list, the rest to another
+__global__ void k_gather_pairs(const int *perm, const int *po, const int *pi, int64_t n0, int64_t n, int *out0, int *in0,
+                               int *out1, int *in1) {
     const int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (d >= n) return;
     const int e = perm[d];
-    g_out[d] = po[e];
-    g_in[d] = pi[e];
+    (d < n0 ? out0 + d : out1 + (d - n0))[0] = po[e];
+    (d < n0 ? in0 + d : in1 + (d - n0))[0] = pi[e];
 }
 
-
-// The M2L pairs of a tree with their operator class as key; with flags set
-// (bit 0: the cell holds charges, bit 1: panels) only those whose source has
-// `src_bit` and whose target has `tgt_bit`.  FILL = false counts them per target.
-template <bool FILL>
-__global__ void k_m2l_pairs(const int *m2l_off, int first, int last, const int *m2l_src, const int *m2l_ofs,
-                            const unsigned char *flags, int src_bit, int tgt_bit, const int *off, int *cnt, int *out,
-                            int *in, int *key) {
-    const int t = first + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= last || (flags && !(flags[t] & tgt_bit))) return;
-    int n = FILL ? off[t] : 0;
-    for (int e = m2l_off[t]; e < m2l_off[t + 1]; ++e) {
-        const int s = m2l_src[e];
-        if (flags && !(flags[s] & src_bit)) continue;
-        if (FILL) {
-            out[n] = t;
-            in[n] = s;
-            key[n] = m2l_ofs[e];
-        }
-        ++n;
+// What the cells of a charge tree hold (bit 0: charges, bit 1: panels), from
+// the leaves upwards (flags zero before).
+__global__ void k_cell_flags(TreeView tv, unsigned *flags) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= tv.nleaf) return;
+    const unsigned f = (tv.chg_beg[l + 1] > tv.chg_beg[l] ? 1u : 0u) |
+                       (tv.cen_beg[l + 1] > tv.cen_beg[l] || tv.qp_beg[l + 1] > tv.qp_beg[l] ? 2u : 0u);
+    for (int c = tv.leaf0 + l; c >= 0 && f != 0; c = tv.parent[c]) {
+        if ((flags[c] & f) == f) break;  // its ancestors have (or are getting) these bits from another leaf
+        atomicOr(flags + c, f);
     }
-    if (!FILL) cnt[t] = n;
+}
+
+// The M2L pairs of a tree with their operator class as key, a warp per target
+// cell (a charge tree's cells have up to 875 partners: one thread a cell took
+// 0.5 ms).  With flags, two lists one behind the other: charges to panels (the
+// source holds charges, the target panels), then panels to charges (keys ncls +
+// class).  FILL = false counts a target's pairs into cnt[list][ncell + 1]; FILL
+// writes the lists l0 .. l1 - 1 in order, from their offsets less `base` on.
+constexpr int PAIR_THREADS = 256;
+template <bool FILL>
+__global__ void __launch_bounds__(PAIR_THREADS)
+k_m2l_pairs(const int *m2l_off, int first, int last, const int *m2l_src, const int *m2l_ofs, int ncls,
+            const unsigned *flags, int l0, int l1, const int *off, int base, int *cnt, int *out, int *in, int *key) {
+    const int t = first + (int)((blockIdx.x * (int64_t)PAIR_THREADS + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (t >= last) return;
+    const int stride = last + 1;  // last = ncell
+    const int b = m2l_off[t], e = m2l_off[t + 1];
+    const unsigned ft = flags ? flags[t] : 0u;
+    int n[2] = {0, 0};
+    if (FILL)
+        for (int l = l0; l < l1; ++l) n[l] = off[l * stride + t] - base;
+    for (int i0 = b; i0 < e; i0 += 32) {
+        const int i = i0 + lane;
+        const int s = i < e ? m2l_src[i] : 0;
+        const unsigned fs = flags && i < e ? flags[s] : 0u;
+        for (int l = l0; l < l1; ++l) {
+            const bool take = i < e && (!flags || ((fs >> l & 1u) && (ft >> (1 - l) & 1u)));
+            const unsigned w = __ballot_sync(0xffffffffu, take);
+            if (FILL && take) {
+                const int d = n[l] + __popc(w & ((1u << lane) - 1u));
+                out[d] = t;
+                in[d] = s;
+                key[d] = l * ncls + m2l_ofs[i];
+            }
+            n[l] += __popc(w);
+        }
+    }
+    if (!FILL && lane == 0)
+        for (int l = l0; l < l1; ++l) cnt[l * stride + t] = n[l];
 }
 
 // Launch order of the near-field kernel: leaves by decreasing work
@@ -1735,104 +1764,111 @@ static void build_p2p_order(Mesh &m, Tree &t) {
 void build_translation_groups(Mesh &m, Tree &t) {
     cudaStream_t s = m.stream;
     const int L = t.L;
-    build_p2p_order(m, t);
+    // Direct charge sums read none of a charge tree's translations and near
+    // lists; the latter are made for sets so large that they may be refused.
+    const bool unread = &t == &m.tc && charge_direct(m);
+    if (!unread || m.nc + m.nqp >= (1 << 23)) build_p2p_order(m, t);
     t.m2m_chunk0.assign(L + 2, 0);
     t.m2m_nchunk.assign(L + 2, 0);
     t.l2l_chunk0.assign(L + 2, 0);
     t.l2l_nchunk.assign(L + 2, 0);
     for (auto &g : t.m2l) g = Tree::M2LPairs();
-    if (L < 2) return;
+    if (L < 2 || unread) return;
     // host copies of the cell structure (parents, coordinates)
     std::vector<int4> ijk(t.ncell);
     std::vector<int> parent(t.ncell);
     BEM_CUDA(cudaMemcpyAsync(ijk.data(), t.ijk.p, t.ncell * sizeof(int4), cudaMemcpyDeviceToHost, s));
     BEM_CUDA(cudaMemcpyAsync(parent.data(), t.parent.p, t.ncell * sizeof(int), cudaMemcpyDeviceToHost, s));
-    // what each cell of a charge tree holds, from its leaves upwards
-    DArray<unsigned char> flags;
-    if (t.has_chg) {
-        const int n = t.nleaf;
-        std::vector<int> tb(n + 1), qb(n + 1), cb(n + 1);
-        BEM_CUDA(cudaMemcpyAsync(tb.data(), t.cen_beg.p, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
-        BEM_CUDA(cudaMemcpyAsync(qb.data(), t.qp_beg.p, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
-        BEM_CUDA(cudaMemcpyAsync(cb.data(), t.chg_beg.p, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
-        BEM_CUDA(cudaStreamSynchronize(s));
-        std::vector<unsigned char> fl(t.ncell, 0);
-        for (int l = 0; l < n; ++l)
-            fl[t.leaf0 + l] = (cb[l + 1] > cb[l] ? 1 : 0) | (tb[l + 1] > tb[l] || qb[l + 1] > qb[l] ? 2 : 0);
-        for (int c = t.ncell - 1; c > 0; --c) fl[parent[c]] |= fl[c];  // children follow their parents
-        flags.alloc(t.ncell);
-        BEM_CUDA(cudaMemcpyAsync(flags.p, fl.data(), t.ncell, cudaMemcpyHostToDevice, s));
-        BEM_CUDA(cudaStreamSynchronize(s));
-    }
     // M2L pairs grouped by offset class on the device: a stable radix sort of
     // the pair indices (target-major list order) by class, the pairs gathered
     // into that order, and only the per-class counts copied to the host to cut
     // the classes into chunks.  A charge tree gets a list per direction of its
-    // passes, without the pairs that carry nothing: of 8 molecules of 81,920
-    // panels and 2,000 charges, the solve with its potential 22.5 -> 19.2 ms.
+    // passes, without the pairs that carry nothing (of 8 molecules of 81,920
+    // panels and 2,000 charges, the solve with its potential 22.5 -> 19.2 ms);
+    // both go through one sort (bem_set_charges of 2,000 charges on 81,920 panels
+    // 5.7 ms with one list of all pairs, 6.3 with two sorts, 4.8 this way; 4,000
+    // charges on 11,520 panels, most pairs in both lists, 2.3, 2.9 and 2.5).
+    std::vector<std::vector<int4>> up;
     const int64_t nm = t.nm2l;
-    const int ncls = m2l_classes(t.ws);
-    int cls_bits = 0;
-    while ((1 << cls_bits) < ncls) ++cls_bits;
+    const int ncls = m2l_classes(t.ws), nlist = t.has_chg ? 2 : 1;
     const int first = t.lvl_off[2], last = t.ncell;
-    const int kinds[2] = {Tree::M2L_CHG_TO_PANEL, Tree::M2L_PANEL_TO_CHG}, all[1] = {Tree::M2L_ALL};
-    for (int q = 0; nm > 0 && q < (t.has_chg ? 2 : 1); ++q) {
-        const int kind = t.has_chg ? kinds[q] : all[q];
-        Tree::M2LPairs &g = t.m2l[kind];
-        const int sb = kind == Tree::M2L_CHG_TO_PANEL ? 1 : 2, tb = 3 - sb;
-        const int nb = cdiv(last - first, 256);
-        DArray<int> po, pi, key, idx, key_s, perm, dcnt, c, off;
-        int64_t nv = nm;
+    if (nm > 0) {
+        const int nb = cdiv((int64_t)(last - first) * 32, PAIR_THREADS), nc1 = t.ncell + 1;
+        DArray<int> small, big;  // per cell and class: flags | counts | offsets | pairs of a class; per pair
+        small.alloc((size_t)(t.has_chg ? t.ncell + 4 * (size_t)nc1 : 0) + nlist * ncls);
+        int *const dcnt = small.p, *const cnt = dcnt + nlist * ncls, *const off = cnt + 2 * nc1;
+        unsigned *const flags = t.has_chg ? reinterpret_cast<unsigned *>(off + 2 * nc1) : nullptr;
+        BEM_CUDA(cudaMemsetAsync(small.p, 0, small.n * sizeof(int), s));
+        int64_t nv = nm, n0 = nm;  // pairs, pairs of the first list
         const int *offp = t.m2l_off.p;
         if (t.has_chg) {
-            c.alloc(t.ncell + 1);
-            off.alloc(t.ncell + 1);
-            BEM_CUDA(cudaMemsetAsync(c.p, 0, (t.ncell + 1) * sizeof(int), s));
-            k_m2l_pairs<false><<<nb, 256, 0, s>>>(t.m2l_off.p, first, last, t.m2l_src.p, t.m2l_ofs.p, flags.p, sb, tb,
-                                                nullptr, c.p, nullptr, nullptr, nullptr);
+            k_cell_flags<<<cdiv(t.nleaf, 256), 256, 0, s>>>(view(t), flags);
             BEM_CHECK_LAUNCH();
-            exclusive_scan_int(c.p, off.p, t.ncell + 1, s);
-            int n = 0;
-            BEM_CUDA(cudaMemcpyAsync(&n, off.p + t.ncell, sizeof(int), cudaMemcpyDeviceToHost, s));
+            k_m2l_pairs<false><<<nb, PAIR_THREADS, 0, s>>>(t.m2l_off.p, first, last, t.m2l_src.p, t.m2l_ofs.p, ncls, flags,
+                                                         0, 2, nullptr, 0, cnt, nullptr, nullptr, nullptr);
+            BEM_CHECK_LAUNCH();
+            exclusive_scan_int(cnt, off, 2 * nc1, s);
+            int n[2] = {0, 0};
+            BEM_CUDA(cudaMemcpyAsync(&n[0], off + t.ncell, sizeof(int), cudaMemcpyDeviceToHost, s));
+            BEM_CUDA(cudaMemcpyAsync(&n[1], off + nc1 + t.ncell, sizeof(int), cudaMemcpyDeviceToHost, s));
             BEM_CUDA(cudaStreamSynchronize(s));
-            nv = n;
-            offp = off.p;
+            n0 = n[0];
+            nv = n[1];
+            offp = off;
         }
-        if (nv == 0) continue;
-        po.alloc(nv);
-        pi.alloc(nv);
-        key.alloc(nv);
-        idx.alloc(nv);
-        key_s.alloc(nv);
-        perm.alloc(nv);
-        dcnt.alloc(ncls);
-        k_m2l_pairs<true><<<nb, 256, 0, s>>>(t.m2l_off.p, first, last, t.m2l_src.p, t.m2l_ofs.p,
-                                           t.has_chg ? flags.p : nullptr, sb, tb, offp, nullptr, po.p, pi.p, key.p);
-        BEM_CHECK_LAUNCH();
-        k_iota<<<cdiv(nv, 256), 256, 0, s>>>(idx.p, nv);
-        BEM_CHECK_LAUNCH();
-        sort_pairs_int(key.p, idx.p, key_s.p, perm.p, nv, cls_bits, s);
-        BEM_CUDA(cudaMemsetAsync(dcnt.p, 0, ncls * sizeof(int), s));
-        k_class_count<<<cdiv(nv, 256), 256, 0, s>>>(key.p, nv, dcnt.p);
-        BEM_CHECK_LAUNCH();
-        std::vector<int> cnt(ncls, 0);
-        BEM_CUDA(cudaMemcpyAsync(cnt.data(), dcnt.p, ncls * sizeof(int), cudaMemcpyDeviceToHost, s));
-        g.out.alloc(nv);
-        g.in.alloc(nv);
-        k_gather_pairs<<<cdiv(nv, 256), 256, 0, s>>>(perm.p, po.p, pi.p, nv, g.out.p, g.in.p);
-        BEM_CHECK_LAUNCH();
-        BEM_CUDA(cudaStreamSynchronize(s));
-        std::vector<int4> chunks;
-        int64_t b0 = 0;
-        for (int o = 0; o < ncls; ++o) {
-            for (int64_t b = b0; b < b0 + cnt[o]; b += TR_BN_M2L)
-                chunks.push_back(make_int4(o, (int)b, (int)std::min<int64_t>(TR_BN_M2L, b0 + cnt[o] - b), 0));
-            b0 += cnt[o];
+        // one sort for both lists while launches count, not the memory of a sort
+        const bool together = nlist == 2 && nv <= (1 << 24);
+        for (int l0 = 0, l1; l0 < nlist; l0 = l1) {
+            l1 = together ? nlist : l0 + 1;
+            const int64_t base = l0 == 0 ? 0 : n0, n = (l1 == nlist ? nv : n0) - base;
+            if (n == 0) continue;
+            big.alloc((size_t)6 * n);
+            int *const po = big.p, *const pi = po + n, *const key = pi + n, *const idx = key + n, *const key_s = idx + n,
+                      *const perm = key_s + n;
+            k_m2l_pairs<true><<<nb, PAIR_THREADS, 0, s>>>(t.m2l_off.p, first, last, t.m2l_src.p, t.m2l_ofs.p, ncls, flags,
+                                                        l0, l1, offp, (int)base, nullptr, po, pi, key);
+            BEM_CHECK_LAUNCH();
+            k_iota<<<cdiv(n, 256), 256, 0, s>>>(idx, n);
+            BEM_CHECK_LAUNCH();
+            int bits = 0;
+            while ((1 << bits) < l1 * ncls) ++bits;
+            sort_pairs_int(key, idx, key_s, perm, n, bits, s);
+            k_class_count<<<cdiv(n, 256), 256, 0, s>>>(key, n, dcnt);
+            BEM_CHECK_LAUNCH();
+            std::vector<int> cls(nlist * ncls, 0);
+            BEM_CUDA(cudaMemcpyAsync(cls.data(), dcnt, cls.size() * sizeof(int), cudaMemcpyDeviceToHost, s));
+            Tree::M2LPairs *g[2];
+            for (int l = l0; l < l1; ++l) {
+                g[l] = &t.m2l[!t.has_chg ? Tree::M2L_ALL : (l == 0 ? Tree::M2L_CHG_TO_PANEL : Tree::M2L_PANEL_TO_CHG)];
+                g[l]->out.alloc(l == 0 ? n0 : nv - n0);
+                g[l]->in.alloc(l == 0 ? n0 : nv - n0);
+            }
+            Tree::M2LPairs &ga = *g[l0], &gb = *g[l1 - 1];
+            k_gather_pairs<<<cdiv(n, 256), 256, 0, s>>>(perm, po, pi, together ? n0 : n, n, ga.out.p, ga.in.p, gb.out.p,
+                                                      gb.in.p);
+            BEM_CHECK_LAUNCH();
+            BEM_CUDA(cudaStreamSynchronize(s));
+            for (int l = l0; l < l1; ++l) {
+                std::vector<int4> chunks;
+                int64_t b0 = 0;
+                for (int o = 0; o < ncls; ++o) {
+                    const int64_t e = b0 + cls[l * ncls + o];
+                    for (int64_t b = b0; b < e; b += TR_BN_M2L)
+                        chunks.push_back(make_int4(o, (int)b, (int)std::min<int64_t>(TR_BN_M2L, e - b), 0));
+                    b0 = e;
+                }
+                if (chunks.empty()) continue;
+                std::vector<int4> sup = tc_items(chunks);
+                g[l]->nchunk = (int)chunks.size();
+                g[l]->nsuper = (int)sup.size();
+                g[l]->chunk.alloc(chunks.size());
+                g[l]->super.alloc(sup.size());
+                BEM_CUDA(cudaMemcpyAsync(g[l]->chunk.p, chunks.data(), chunks.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+                BEM_CUDA(cudaMemcpyAsync(g[l]->super.p, sup.data(), sup.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+                up.push_back(std::move(chunks));  // read until the stream is synchronised below
+                up.push_back(std::move(sup));
+            }
         }
-        g.nchunk = (int)chunks.size();
-        g.chunk.alloc(chunks.size());
-        BEM_CUDA(cudaMemcpyAsync(g.chunk.p, chunks.data(), chunks.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-        build_tc_super(g, chunks, s);  // synchronises: the copies above are done
     }
     std::vector<int4> chunks;
     // M2M (out parent, in child) and L2L (out child, in parent) per child level

@@ -409,7 +409,7 @@ constexpr int TC_TABLE_DIM = 128;
 __host__ __device__ inline int tc_table_index(int in, int out) {
     return ((in >> 2) * TC_TABLE_DIM + out) * 4 + (in & 3);
 }
-void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cudaStream_t s);
+std::vector<int4> tc_items(const std::vector<int4> &chunks_m2l);
 void m2l_tc(Mesh &m, const Tree &t, const Tree::M2LPairs &g, const float *M, float *L, bool timed = false);
 bool use_tc_m2l(const Mesh &m);
 // stride of the expansions' rows: row_stride, or 32 values (rows on whole

@@ -526,7 +526,7 @@ size_t tc_smem_bytes() { return 1024 + (size_t)TC_NS * TC_STAGE_BYTES + (size_t)
 // Work items of the persistent kernel: (offset class, first pair, number of
 // pairs), up to TC_CHUNKS_PER_ITEM consecutive 64-pair chunks of one class
 // (tiles of 128 pairs), largest first.
-void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cudaStream_t s) {
+std::vector<int4> tc_items(const std::vector<int4> &chunks_m2l) {
     std::vector<int4> sup;
     int i = 0;
     const int n = (int)chunks_m2l.size();
@@ -537,11 +537,7 @@ void build_tc_super(Tree::M2LPairs &g, const std::vector<int4> &chunks_m2l, cuda
         i = j;
     }
     std::stable_sort(sup.begin(), sup.end(), [](const int4 &a, const int4 &b) { return a.z > b.z; });
-    g.super.alloc(sup.size());
-    g.nsuper = (int)sup.size();
-    if (!sup.empty())
-        BEM_CUDA(cudaMemcpyAsync(g.super.p, sup.data(), sup.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-    BEM_CUDA(cudaStreamSynchronize(s));
+    return sup;
 }
 
 // L (levels >= 2, cleared by the pass) += sum over the M2L pairs of T_o M_s.
