@@ -410,8 +410,7 @@ static void rhs_sorted(Mesh &m, double *b_s) {
         BEM_CUDA(cudaMemsetAsync(b_s, 0, m.np * sizeof(double), m.stream));
         return;
     }
-    charge_pass(m, SRC_CHARGE, m.opt.galerkin ? TGT_QUAD_DN : TGT_CEN_DN, nullptr, m.zs.p);
-    axpby(m, -m.ehat, m.zs.p, 0.0, m.zs.p, b_s, m.np);
+    charge_pass(m, SRC_CHARGE, m.opt.galerkin ? TGT_QUAD_DN : TGT_CEN_DN, nullptr, b_s, -m.ehat);
 }
 
 int bem_rhs(bem_mesh *m, double *b) {
@@ -481,8 +480,7 @@ static double energy_sorted(Mesh &m, const double *sig_s, double *phi_user) {
     if (phi_user) {
         // phi_reac = (C sigma) / eps_in in the caller's charge order
         OutArg o = dev_out(m, phi_user, m.nc, m.io_b);
-        axpby(m, 1.0 / m.eps_in, phi_s, 0.0, phi_s, m.ys.p, m.nc);
-        scatter_f64(m.ys.p, m.chg_perm.p, o.dev, m.nc, m.stream);
+        scatter_scaled(1.0 / m.eps_in, phi_s, m.chg_perm.p, o.dev, m.nc, m.stream);
         finish_out(m, o);
     }
     return dG;
@@ -514,10 +512,7 @@ int bem_bibee(bem_mesh *m, int variant, double *sigma_hat, double *dG) {
         // sigma_hat = -Ehat / (1 + Ehat lambda) (B q)
         const double f = -m->ehat / (1.0 + m->ehat * lam);
         if (m->nc == 0) BEM_CUDA(cudaMemsetAsync(m->xs.p, 0, m->np * sizeof(double), m->stream));
-        else {
-            charge_pass(*m, SRC_CHARGE, m->opt.galerkin ? TGT_QUAD_DN : TGT_CEN_DN, nullptr, m->zs.p);
-            axpby(*m, f, m->zs.p, 0.0, m->zs.p, m->xs.p, m->np);
-        }
+        else charge_pass(*m, SRC_CHARGE, m->opt.galerkin ? TGT_QUAD_DN : TGT_CEN_DN, nullptr, m->xs.p, f);
         if (sigma_hat) {
             OutArg o = dev_out(*m, sigma_hat, m->np, m->io_b);
             scatter_f64(m->xs.p, m->cen_perm.p, o.dev, m->np, m->stream);

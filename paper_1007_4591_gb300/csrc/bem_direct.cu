@@ -24,6 +24,8 @@
 
 namespace bem {
 
+void axpby(Mesh &m, double a, const double *x, double b, const double *y, double *out, int64_t n);
+
 constexpr int DIRECT_THREADS = 256;  // FP64 kernel
 constexpr int DIRECT_TILE = 256;     // sources per tile of either kernel
 
@@ -321,12 +323,13 @@ void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, flo
     }
 }
 
-// out[i] = scale x the sum of the splits' parts: `group` consecutive splits in
+// out[i] = mul x scale x the sum of the splits' parts: `group` consecutive splits in
 // T (as if one CTA had summed their sources), then FP64 over the groups, shared
 // by `lanes` threads (one thread loading 280 splits in turn took 20 us); n
 // values, one to four of them a target.
 template <class T>
-__global__ void k_direct_reduce(const T *part, int nsplit, int group, int64_t n, double scale, int lanes, double *out) {
+__global__ void k_direct_reduce(const T *part, int nsplit, int group, int64_t n, double scale, double mul, int lanes,
+                                double *out) {
     __shared__ double sh[256];
     const int per = blockDim.x / lanes, t = threadIdx.x % per, lane = threadIdx.x / per;
     const int64_t i = blockIdx.x * (int64_t)per + t;
@@ -341,22 +344,23 @@ __global__ void k_direct_reduce(const T *part, int nsplit, int group, int64_t n,
     __syncthreads();
     if (lane == 0 && i < n) {
         for (int l = 1; l < lanes; ++l) s += sh[l * per + t];
-        out[i] = scale * s;
+        const double v = scale * s;
+        out[i] = mul == 1.0 ? v : mul * v + 0.0 * v;  // as axpby does (a value that is not finite gives NaN)
     }
 }
 
 template <class T>
-void direct_reduce(const T *part, int nsplit, int group, int64_t n, int no, double *out, cudaStream_t s) {
+void direct_reduce(const T *part, int nsplit, int group, int64_t n, int no, double *out, cudaStream_t s, double mul) {
     const int ng = (nsplit + group - 1) / group, lanes = ng > 128 ? 32 : (ng > 16 ? 8 : 1);
-    k_direct_reduce<T><<<cdiv(n * no, 256 / lanes), 256, 0, s>>>(part, nsplit, group, n * no, 1.0 / FOUR_PI, lanes, out);
+    k_direct_reduce<T><<<cdiv(n * no, 256 / lanes), 256, 0, s>>>(part, nsplit, group, n * no, 1.0 / FOUR_PI, mul, lanes, out);
     BEM_CHECK_LAUNCH();
 }
-template void direct_reduce<float>(const float *, int, int, int64_t, int, double *, cudaStream_t);
-template void direct_reduce<double>(const double *, int, int, int64_t, int, double *, cudaStream_t);
+template void direct_reduce<float>(const float *, int, int, int64_t, int, double *, cudaStream_t, double);
+template void direct_reduce<double>(const double *, int, int, int64_t, int, double *, cudaStream_t, double);
 
-// out_j = sum_q (qw_jq / A_j) v_jq: the rule's average over panel j
+// out_j = mul sum_q (qw_jq / A_j) v_jq: the rule's average over panel j
 __global__ void k_panel_avg(const double *v, const int *qp_of_panel, const double *qw, const double *area,
-                            int nq, int64_t np, double *out) {
+                            int nq, int64_t np, double mul, double *out) {
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= np) return;
     double a = 0.0;
@@ -364,12 +368,12 @@ __global__ void k_panel_avg(const double *v, const int *qp_of_panel, const doubl
         const int k = qp_of_panel[j * nq + q];
         a += qw[k] * v[k];
     }
-    out[j] = a / area[j];
+    const double r = a / area[j];
+    out[j] = mul == 1.0 ? r : mul * r + 0.0 * r;
 }
 
 template <class T>
-static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out,
-                        DArray<T> &part) {
+static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out, DArray<T> &part, double mul) {
     cudaStream_t s = m.stream;
     const int64_t ntgt = (tk == TGT_CEN_DN) ? m.np : ((tk == TGT_QUAD_DN || tk == TGT_QUAD_PHI) ? m.nqp : m.nc);
     // Galerkin rows: the values at the quadrature points, then the rule's
@@ -443,10 +447,10 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
         else if (tnrm) go(k_direct<SRC_CHARGE, TGT_CEN_DN>);
         else go(k_direct<SRC_CHARGE, TGT_CHG_PHI>);
     }
-    direct_reduce<T>(part.p, nsplit, group, ntgt, 1, out, s);
+    direct_reduce<T>(part.p, nsplit, group, ntgt, 1, out, s, tk == TGT_QUAD_DN ? 1.0 : mul);
     if (tk == TGT_QUAD_DN) {
         k_panel_avg<<<cdiv(m.np, 256), 256, 0, s>>>(out, m.qp_of_panel.p, m.qw64.p, m.area64.p, (int)m.nq,
-                                                    m.np, final_out);
+                                                    m.np, mul, final_out);
         BEM_CHECK_LAUNCH();
     }
 }
@@ -485,9 +489,9 @@ void build_ctq(Mesh &m) {
     m.ctq_ok = true;
 }
 
-void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out) {
-    if (m.opt.precision == BEM_MIXED) direct_impl<float>(m, sk, tk, dens, out, m.dpart_f);
-    else direct_impl<double>(m, sk, tk, dens, out, m.dpart_d);
+void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out, double mul) {
+    if (m.opt.precision == BEM_MIXED) direct_impl<float>(m, sk, tk, dens, out, m.dpart_f, mul);
+    else direct_impl<double>(m, sk, tk, dens, out, m.dpart_d, mul);
 }
 
 bool charge_direct(const Mesh &m) {
@@ -496,9 +500,13 @@ bool charge_direct(const Mesh &m) {
     return (double)m.nc * (double)m.nqp <= 4e10;
 }
 
-void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out) {
-    if (charge_direct(m)) direct_pass(m, sk, tk, dens, out);
-    else fmm_pass(m, m.tc, sk, tk, dens, out, false);
+void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out, double mul) {
+    if (charge_direct(m)) {
+        direct_pass(m, sk, tk, dens, out, mul);
+        return;
+    }
+    fmm_pass(m, m.tc, sk, tk, dens, out, false);
+    if (mul != 1.0) axpby(m, mul, out, 0.0, out, out, tk == TGT_CHG_PHI ? m.nc : m.np);
 }
 
 }  // namespace bem

@@ -440,9 +440,9 @@ bool is_near_field_kernel(const void *func);
 // Products between the charges and the surface (B q, C sigma): the fast
 // multipole pass on the charge tree, or the direct sum over all pairs,
 // following opt.charge_mode.
-void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out);
+void charge_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out, double mul = 1.0);
 bool charge_direct(const Mesh &m);
-void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out);
+void direct_pass(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out, double mul = 1.0);
 void build_ctq(Mesh &m);
 // the adjoint gradients' vectors, kept with the mesh from its first gradient on:
 // (phi, grad) of C sigma and of B^T lam, the gradients, lam
@@ -475,10 +475,10 @@ inline double parts_limit(const Mesh &m) { return 64.0 * (double)m.np; }
 inline int splits_limit(const Mesh &m, int64_t values) { return (int)std::min(65535.0, parts_limit(m) / (double)values); }
 // part[split][target] (x 4 with the gradient), split s over the sources [s chunk, (s + 1) chunk)
 void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, float *part);
-// out[n][no] = 1/(4 pi) x the sum over the splits of part[split][n][no], each
+// out[n][no] = mul/(4 pi) x the sum over the splits of part[split][n][no], each
 // `group` consecutive splits added in T first
 template <class T>
-void direct_reduce(const T *part, int nsplit, int group, int64_t n, int no, double *out, cudaStream_t s);
+void direct_reduce(const T *part, int nsplit, int group, int64_t n, int no, double *out, cudaStream_t s, double mul = 1.0);
 // per panel, the weighted sum of its quadrature points' values
 void panel_wsum(Mesh &m, const double *v, double *out);
 double energy_from_ctq(Mesh &m, const double *sig_s);
@@ -490,6 +490,7 @@ void matvec_t_sorted(Mesh &m, const double *xs, double *ys);
 void exclusive_scan_int(const int *in, int *out, int n, cudaStream_t s);
 void gather_f64(const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s);
 void scatter_f64(const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s);
+void scatter_scaled(double a, const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s);
 void scatter_rows3(const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s);
 
 }  // namespace bem

@@ -24,6 +24,10 @@ __global__ void k_scatter(const double *src, const int *perm, double *dst, int64
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) dst[perm[i]] = src[i];
 }
+__global__ void k_scatter_scaled(double a, const double *src, const int *perm, double *dst, int64_t n) {
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) dst[perm[i]] = a * src[i] + 0.0 * src[i];  // as axpby does (a value that is not finite gives NaN)
+}
 __global__ void k_scatter3(const double *src, const int *perm, double *dst, int64_t n) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -39,6 +43,11 @@ void gather_f64(const double *src, const int *perm, double *dst, int64_t n, cuda
 }
 void scatter_f64(const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s) {
     k_scatter<<<cdiv(n, 256), 256, 0, s>>>(src, perm, dst, n);
+    BEM_CHECK_LAUNCH();
+}
+void scatter_scaled(double a, const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s) {
+    if (n <= 0) return;
+    k_scatter_scaled<<<cdiv(n, 256), 256, 0, s>>>(a, src, perm, dst, n);
     BEM_CHECK_LAUNCH();
 }
 void scatter_rows3(const double *src, const int *perm, double *dst, int64_t n, cudaStream_t s) {
