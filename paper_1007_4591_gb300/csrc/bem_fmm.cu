@@ -2152,7 +2152,12 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
         launch_near(m.stream2);
         BEM_CUDA(cudaEventRecord(m.ev_join, m.stream2));
     };
-    if (conc && (dense || !far)) fork_near();
+    // In a captured graph both branches are ready at once and the near field
+    // would take the SMs first: there it forks after the clearing kernel (graph
+    // replay, 8,000 panels 105 us, 103 to 141 forked at the start; 15,680 panels
+    // 168 and 185 to 222; 81,920 panels 267 and 266).
+    const bool late = dense && m.capturing;
+    if (conc && ((dense && !late) || !far)) fork_near();
     if (far) {
         T *M = B::M(m), *L = B::L(m);
         const int cs = cell_stride(m);
@@ -2160,6 +2165,7 @@ static void run_pass(Mesh &m, const Tree &t, SrcKind sk, TgtKind tk, const doubl
         const size_t trsm = translate_smem<T, TR_BN_M2L>();
         if (dense) set_smem<T>(k_translate<T, TR_BN_M2L, TR_THREADS>, trsm);
         if (dense) clear_expansions<T>(m, t, M, L, cs);
+        if (conc && late) fork_near();
         // P2M
         p2m_leaves<T>(tv, t.nleaf, sk, srec, qpanel, dens, p, cs, inv_h, M, s);
         ev_rec(m, timed, 1);
