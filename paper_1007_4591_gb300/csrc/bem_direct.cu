@@ -296,7 +296,8 @@ void direct_partials(Mesh &m, const DirectSum &d, int64_t chunk, int nsplit, flo
     float4 *rec;
     size_t room;
     record_space(m, d.to_quad_values, rec, room);
-    const int64_t seg = (int64_t)(room / rs / DIRECT_TILE * DIRECT_TILE);
+    // (at most 32,768 splits a launch)
+    const int64_t seg = std::min((int64_t)(room / rs / DIRECT_TILE), (int64_t)1 << 15) * DIRECT_TILE;
     if (seg == 0) throw Error(BEM_ECUDA, "direct sums: no room for a tile of records");
     const double ox = m.root_min[0] + 0.5 * m.side, oy = m.root_min[1] + 0.5 * m.side,
                  oz = m.root_min[2] + 0.5 * m.side;
@@ -351,7 +352,7 @@ __global__ void k_direct_reduce(const T *part, int nsplit, int group, int64_t n,
 
 template <class T>
 void direct_reduce(const T *part, int nsplit, int group, int64_t n, int no, double *out, cudaStream_t s, double mul) {
-    const int ng = (nsplit + group - 1) / group, lanes = ng > 128 ? 32 : (ng > 16 ? 8 : 1);
+    const int ng = (nsplit + group - 1) / group, lanes = ng > 1024 ? 256 : (ng > 128 ? 32 : (ng > 16 ? 8 : 1));
     k_direct_reduce<T><<<cdiv(n * no, 256 / lanes), 256, 0, s>>>(part, nsplit, group, n * no, 1.0 / FOUR_PI, mul, lanes, out);
     BEM_CHECK_LAUNCH();
 }
@@ -390,23 +391,19 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
         return;
     }
     const int tblocks = cdiv(ntgt, DIRECT_THREADS);
-    // enough CTAs to fill the GPU, splits of at least 512 sources: 16 CTAs per
-    // SM, or for the potential of the quadrature points at the charges in FP32
-    // (few targets, many splits) four waves of its kernel (2,000 charges,
-    // 573,440 points: 484 us against 531 in one wave)
-    constexpr bool F32 = std::is_same<T, float>::value;
-    const int ctas = F32 && sk == SRC_QUAD ? 4 * 10 * 152 : 2432;
-    int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, 512), std::max(1, ctas / tblocks)));
-    if (F32 && sk == SRC_QUAD)
-        nsplit = std::min(nsplit, std::max({splits_limit(m, ntgt), 2432 / tblocks, 1}));
+    // enough CTAs to fill the GPU about twice (16 per SM), splits of at least 512 sources
+    int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, 512), std::max(1, 2432 / tblocks)));
     nsplit = std::min(nsplit, 65535);
     int64_t chunk = (nsrc + nsplit - 1) / nsplit;
     chunk = ((chunk + DIRECT_THREADS - 1) / DIRECT_THREADS) * DIRECT_THREADS;
-    // FP32 sums over the charges: a CTA per tile of a split, the split's tiles
-    // added in order by the reduction (the sums a CTA per split gives, in
-    // shorter CTAs: 81,920 targets, 2,000 charges are 1.2 waves of splits)
+    // FP32: a CTA per tile of a split, the split's tiles added in order by the
+    // reduction: bit for bit the sums that a CTA per split gives, in shorter CTAs
+    // (81,920 targets, 2,000 charges are 1.2 waves of splits; 100 targets, 28.7M
+    // points 1.6: 4.30 ms, 5.08 with a CTA per split)
+    constexpr bool F32 = std::is_same<T, float>::value;
     int group = 1;
-    if (F32 && sk == SRC_CHARGE && (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= parts_limit(m)) {
+    if (F32 && chunk <= 64 * DIRECT_TILE &&
+        (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= (sk == SRC_QUAD ? 1.5 : 1.0) * parts_limit(m)) {
         group = (int)(chunk / DIRECT_TILE);
         chunk = DIRECT_TILE;
     }

@@ -469,7 +469,7 @@ double *quad_values(Mesh &m);
 // for quad_values and a tile of source records beside them
 size_t direct_space(const Mesh &m);
 // FP32 partial sums that a direct sum may keep: 64 a panel (256 bytes, of some
-// 2,500 a mesh holds for it), where a few waves of CTAs need fewer anyway
+// 2,500 a mesh holds for it; half as many again for the potential at the charges)
 inline double parts_limit(const Mesh &m) { return 64.0 * (double)m.np; }
 // the splits of a sum of `values` numbers that stay below it
 inline int splits_limit(const Mesh &m, int64_t values) { return (int)std::min(65535.0, parts_limit(m) / (double)values); }

@@ -63,6 +63,27 @@ def test_single_translations_keep_their_bits(pkg, golden, p, diagonal):
     assert far_field(pkg, p, diagonal).tolist() == ref
 
 
+POTENTIALS = {"small-s4, 60 charges": lambda: synth.small_molecule(4, n_charges=60),
+              "globular-s6, 700 charges": lambda: synth.globular(6, n_charges=700)}
+
+
+def potential(pkg, name):
+    """C s at the charges for a fixed density: the right-hand side's, which no
+    multipole pass has touched."""
+    m = POTENTIALS[name]()
+    with pkg.Mesh(m.panels, m.charges, m.eps_in, m.eps_out, charge_mode=pkg.BEM_CHARGE_DIRECT) as g:
+        return g.energy(g.rhs(), want_phi=True)[1].cpu().numpy()[::20]
+
+
+@pytest.mark.parametrize("name", sorted(POTENTIALS))
+def test_direct_sums_keep_their_bits(pkg, golden, name):
+    """All-pairs sums have no order of arrival: normal field and potential, tile
+    by tile in splits of the same length.  The last FP64 sum over the splits may
+    be shared out differently (2^-52 a term, at most some thousands)."""
+    ref = np.array([float.fromhex(v) for v in golden["potential"][name]])
+    assert np.abs(potential(pkg, name) / ref - 1).max() < 1e-12
+
+
 @pytest.mark.parametrize("name", sorted(MOLECULES))
 def test_energy_from_call_to_call(pkg, golden, name):
     """200 calls before the multipoles were split inside the M2L kernel: mean as
