@@ -449,10 +449,9 @@ def run_ours(args):
         near_k.append(pkg.bem_last_near_ms(mesh.h))
     pkg.bem_set_profiling(mesh.h, False)
     ph = {k: float(np.mean([d[k] for d in phases])) for k in phases[0]}
-    # the M2L phase holds the multipole split and the tensor-core kernel
-    # (zeros when the product has no tensor-core M2L: then the whole phase is
-    # the SIMT kernel); the P2P phase the strength records and the
-    # near-field kernel
+    # the M2L phase holds the tensor-core kernel (which splits the multipoles
+    # itself: the "split" entry is near zero), or the SIMT kernel (both entries
+    # zero); the P2P phase the strength records and the near-field kernel
     mk = {k: float(np.mean([d[k] for d in m2l_k])) for k in m2l_k[0]}
     nk = {k: float(np.mean([d[k] for d in near_k])) for k in near_k[0]}
     t_m2l = mk["tc"] if mk["tc"] > 0 else ph["m2l"]
@@ -534,7 +533,7 @@ def run_ours(args):
 
     L = info["depth"]
     # gather, source strengths, P2P (with the near-singular table), scatter;
-    # P2M, multipole split, tensor-core M2L, L2P (with the operator's
+    # the clearing kernel, P2M, tensor-core M2L, L2P (with the operator's
     # epilogue) and one M2M and one L2L launch per level from 3 to L (14
     # kernels at L = 5); without a far field, an epilogue kernel instead
     launches_per = 4 + ((4 + 2 * (L - 2)) if L >= 2 else 1)

@@ -267,6 +267,8 @@ def bem_last_phase_ms(h):
 
 
 def bem_last_m2l_ms(h):
+    """Device times of the last profiled tensor-core M2L, ms: "tc" its kernel,
+    "split" near 0 (the kernel splits the multipoles itself)."""
     t = np.zeros(3)
     _check(load_library().bem_last_m2l_ms(h, _ptr(t)), "bem_last_m2l_ms")
     return dict(zip(["split", "tc"], t.tolist()[:2]))

@@ -71,9 +71,10 @@ __device__ __forceinline__ float ex2a(float x) {
     return y;
 }
 __device__ __forceinline__ float rinv3(float r2) { return ex2a(-1.5f * lg2a(r2)); }
-// FP64: the hardware's 20-bit estimate y of r^-1 (relative error d, |d| < 2^-20)
-// corrected by the binomial series of (1 - e)^(-3/2) in e = 1 - r^2 y^2 up to e^2
-// (the next term is below 2^-56): six FP64 operations where rsqrt and its cube
+// FP64: the hardware's 20-bit estimate y of r^-1, corrected by the binomial
+// series of (1 - e)^(-3/2) in e = 1 - r^2 y^2 up to e^2.  |e| was measured below
+// 2^-19.05 over 2^24 values of r^2 in [2^-20, 2^20], so the next term, 35/16 e^3,
+// is below 2^-56.  Six FP64 operations where rsqrt and its cube
 // take eight.  FP64 issue bounds every caller (a pair takes 20.2 issue slots
 // against 21.4), and the error falls from 5.4e-16 to 2.3e-16.
 __device__ __forceinline__ double rinv3(double r2) {
