@@ -373,6 +373,31 @@ __global__ void k_panel_avg(const double *v, const int *qp_of_panel, const doubl
     out[j] = mul == 1.0 ? r : mul * r + 0.0 * r;
 }
 
+// How a sum is cut: splits of `chunk` sources, `group` of them added in T before FP64.
+struct DirectCut {
+    int64_t chunk;
+    int nsplit, group;
+};
+static DirectCut direct_cut(const Mesh &m, bool f32, SrcKind sk, int64_t nsrc, int64_t ntgt) {
+    const int tblocks = cdiv(ntgt, DIRECT_THREADS);
+    // enough CTAs to fill the GPU about twice (16 per SM), splits of at least 512 sources
+    int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, 512), std::max(1, 2432 / tblocks)));
+    nsplit = std::min(nsplit, 65535);
+    int64_t chunk = (nsrc + nsplit - 1) / nsplit;
+    chunk = ((chunk + DIRECT_THREADS - 1) / DIRECT_THREADS) * DIRECT_THREADS;
+    // FP32: a CTA per tile of a split, the split's tiles added in order by the
+    // reduction: bit for bit the sums that a CTA per split gives, in shorter CTAs
+    // (81,920 targets, 2,000 charges are 1.2 waves of splits; 100 targets, 28.7M
+    // points 1.6: 4.30 ms, 5.08 with a CTA per split)
+    int group = 1;
+    if (f32 && chunk <= 64 * DIRECT_TILE &&
+        (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= (sk == SRC_QUAD ? 1.5 : 1.0) * parts_limit(m)) {
+        group = (int)(chunk / DIRECT_TILE);
+        chunk = DIRECT_TILE;
+    }
+    return DirectCut{chunk, (int)((nsrc + chunk - 1) / chunk), group};
+}
+
 template <class T>
 static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, double *out, DArray<T> &part, double mul) {
     cudaStream_t s = m.stream;
@@ -390,24 +415,9 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
         BEM_CUDA(cudaMemsetAsync(final_out, 0, (tk == TGT_QUAD_DN ? m.np : ntgt) * sizeof(double), s));
         return;
     }
-    const int tblocks = cdiv(ntgt, DIRECT_THREADS);
-    // enough CTAs to fill the GPU about twice (16 per SM), splits of at least 512 sources
-    int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, 512), std::max(1, 2432 / tblocks)));
-    nsplit = std::min(nsplit, 65535);
-    int64_t chunk = (nsrc + nsplit - 1) / nsplit;
-    chunk = ((chunk + DIRECT_THREADS - 1) / DIRECT_THREADS) * DIRECT_THREADS;
-    // FP32: a CTA per tile of a split, the split's tiles added in order by the
-    // reduction: bit for bit the sums that a CTA per split gives, in shorter CTAs
-    // (81,920 targets, 2,000 charges are 1.2 waves of splits; 100 targets, 28.7M
-    // points 1.6: 4.30 ms, 5.08 with a CTA per split)
-    constexpr bool F32 = std::is_same<T, float>::value;
-    int group = 1;
-    if (F32 && chunk <= 64 * DIRECT_TILE &&
-        (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= (sk == SRC_QUAD ? 1.5 : 1.0) * parts_limit(m)) {
-        group = (int)(chunk / DIRECT_TILE);
-        chunk = DIRECT_TILE;
-    }
-    nsplit = (int)((nsrc + chunk - 1) / chunk);
+    const DirectCut cut = direct_cut(m, std::is_same<T, float>::value, sk, nsrc, ntgt);
+    const int64_t chunk = cut.chunk;
+    const int nsplit = cut.nsplit, group = cut.group, tblocks = cdiv(ntgt, DIRECT_THREADS);
     const size_t need = (size_t)nsplit * ntgt;
     if (part.n < need) part.alloc(need);
     [[maybe_unused]] const double ox = m.root_min[0] + 0.5 * m.side, oy = m.root_min[1] + 0.5 * m.side,
@@ -478,6 +488,12 @@ void build_ctq(Mesh &m) {
     m.ctq_ok = false;
     if (m.nc == 0 || !charge_direct(m)) return;
     if (m.ctq.n < (size_t)m.np) m.ctq.alloc(m.np);
+    if (m.opt.precision == BEM_MIXED) {  // room for both sums over the charges, not left to the first right-hand side
+        const int64_t nt = m.opt.galerkin ? m.nqp : m.np;
+        const size_t need = std::max((size_t)direct_cut(m, true, SRC_CHARGE, m.nc, nt).nsplit * nt,
+                                     (size_t)direct_cut(m, true, SRC_CHARGE, m.nc, m.nqp).nsplit * m.nqp);
+        if (m.dpart_f.n < need) m.dpart_f.alloc(need);
+    }
     double *psi = quad_values(m);
     direct_pass(m, SRC_CHARGE, TGT_QUAD_PHI, nullptr, psi);
     panel_wsum(m, psi, m.ctq.p);
