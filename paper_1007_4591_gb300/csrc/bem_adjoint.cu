@@ -128,12 +128,26 @@ static void direct_adjoint(Mesh &m, AdjSrc sk, AdjTgt tk, const double *dens, do
     const int tblocks = cdiv(ntgt, ADJ_THREADS);
     // splits of at least 4,096 sources (FP64) or 512 (FP32: a CTA is four warps,
     // and a thousand charges give few blocks of targets)
-    int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, f32 ? 512 : 4096), std::max(1, (f32 ? 4 * 8 * 152 : 1216) / tblocks)));
-    if (f32) nsplit = std::min(nsplit, std::max({splits_limit(m, ntgt * no), std::min(cdiv(nsrc, 4096), 1216 / tblocks), 1}));
-    nsplit = std::min(nsplit, 65535);
-    int64_t chunk = (nsrc + nsplit - 1) / nsplit;
-    chunk = ((chunk + ADJ_THREADS - 1) / ADJ_THREADS) * ADJ_THREADS;
-    nsplit = (int)((nsrc + chunk - 1) / chunk);
+    const int few = std::max(1, std::min(cdiv(nsrc, 4096), 1216 / tblocks));
+    int nsplit = few;
+    if (f32) nsplit = std::max(few, std::min({cdiv(nsrc, 512), 4 * 8 * 152 / tblocks, splits_limit(m, ntgt * no)}));
+    int64_t chunk = 0;
+    auto cut = [&](int n) {
+        n = std::min(n, 65535);
+        chunk = (nsrc + n - 1) / n;
+        chunk = ((chunk + ADJ_THREADS - 1) / ADJ_THREADS) * ADJ_THREADS;
+        nsplit = (int)((nsrc + chunk - 1) / chunk);
+    };
+    cut(nsplit);
+    if (f32 && m.dpart_f.n < (size_t)nsplit * ntgt * no) {
+        try {
+            m.dpart_f.alloc((size_t)nsplit * ntgt * no);
+        } catch (const Error &e) {  // no room for so many splits
+            if (e.code != BEM_ENOMEM) throw;
+            cut(few);
+            m.dpart_f.alloc((size_t)nsplit * ntgt * no);
+        }
+    }
     DirectSum d;
     d.dipole = sk == AS_DIPOLE;
     d.skip_coincident = true;
@@ -149,7 +163,6 @@ static void direct_adjoint(Mesh &m, AdjSrc sk, AdjTgt tk, const double *dens, do
     d.to_quad_values = out == quad_values(m);
     const size_t need = (size_t)nsplit * ntgt * no;
     if (f32) {
-        if (m.dpart_f.n < need) m.dpart_f.alloc(need);
         direct_partials(m, d, chunk, nsplit, m.dpart_f.p);
         direct_reduce(m.dpart_f.p, nsplit, 1, ntgt, no, out, s);
         return;

@@ -373,12 +373,14 @@ __global__ void k_panel_avg(const double *v, const int *qp_of_panel, const doubl
     out[j] = mul == 1.0 ? r : mul * r + 0.0 * r;
 }
 
-// How a sum is cut: splits of `chunk` sources, `group` of them added in T before FP64.
+// How a sum is cut: splits of `chunk` sources, `group` of them added in T before
+// FP64.  With tiles = false a CTA sums a whole split: the same sums from fewer
+// parts, for a device that has no room for more.
 struct DirectCut {
     int64_t chunk;
     int nsplit, group;
 };
-static DirectCut direct_cut(const Mesh &m, bool f32, SrcKind sk, int64_t nsrc, int64_t ntgt) {
+static DirectCut direct_cut(const Mesh &m, bool tiles, SrcKind sk, int64_t nsrc, int64_t ntgt) {
     const int tblocks = cdiv(ntgt, DIRECT_THREADS);
     // enough CTAs to fill the GPU about twice (16 per SM), splits of at least 512 sources
     int nsplit = std::max(1, (int)std::min<int64_t>(cdiv(nsrc, 512), std::max(1, 2432 / tblocks)));
@@ -390,7 +392,7 @@ static DirectCut direct_cut(const Mesh &m, bool f32, SrcKind sk, int64_t nsrc, i
     // (81,920 targets, 2,000 charges are 1.2 waves of splits; 100 targets, 28.7M
     // points 1.6: 4.30 ms, 5.08 with a CTA per split)
     int group = 1;
-    if (f32 && chunk <= 64 * DIRECT_TILE &&
+    if (tiles && chunk <= 64 * DIRECT_TILE &&
         (double)cdiv(nsrc, DIRECT_TILE) * ntgt <= (sk == SRC_QUAD ? 1.5 : 1.0) * parts_limit(m)) {
         group = (int)(chunk / DIRECT_TILE);
         chunk = DIRECT_TILE;
@@ -415,11 +417,19 @@ static void direct_impl(Mesh &m, SrcKind sk, TgtKind tk, const double *dens, dou
         BEM_CUDA(cudaMemsetAsync(final_out, 0, (tk == TGT_QUAD_DN ? m.np : ntgt) * sizeof(double), s));
         return;
     }
-    const DirectCut cut = direct_cut(m, std::is_same<T, float>::value, sk, nsrc, ntgt);
+    DirectCut cut = direct_cut(m, std::is_same<T, float>::value, sk, nsrc, ntgt);
+    if (part.n < (size_t)cut.nsplit * ntgt) {
+        try {
+            part.alloc((size_t)cut.nsplit * ntgt);
+        } catch (const Error &e) {
+            if (e.code != BEM_ENOMEM || cut.group == 1) throw;
+            cut = direct_cut(m, false, sk, nsrc, ntgt);
+            part.alloc((size_t)cut.nsplit * ntgt);
+        }
+    }
     const int64_t chunk = cut.chunk;
-    const int nsplit = cut.nsplit, group = cut.group, tblocks = cdiv(ntgt, DIRECT_THREADS);
-    const size_t need = (size_t)nsplit * ntgt;
-    if (part.n < need) part.alloc(need);
+    const int nsplit = cut.nsplit, group = cut.group;
+    [[maybe_unused]] const int tblocks = cdiv(ntgt, DIRECT_THREADS);
     [[maybe_unused]] const double ox = m.root_min[0] + 0.5 * m.side, oy = m.root_min[1] + 0.5 * m.side,
                                   oz = m.root_min[2] + 0.5 * m.side;
     const double *tpos = (tk == TGT_CEN_DN) ? m.cen64.p : ((tk == TGT_QUAD_DN || tk == TGT_QUAD_PHI) ? m.qpg64.p : m.chgg64.p);
@@ -492,7 +502,13 @@ void build_ctq(Mesh &m) {
         const int64_t nt = m.opt.galerkin ? m.nqp : m.np;
         const size_t need = std::max((size_t)direct_cut(m, true, SRC_CHARGE, m.nc, nt).nsplit * nt,
                                      (size_t)direct_cut(m, true, SRC_CHARGE, m.nc, m.nqp).nsplit * m.nqp);
-        if (m.dpart_f.n < need) m.dpart_f.alloc(need);
+        if (m.dpart_f.n < need) {
+            try {
+                m.dpart_f.alloc(need);
+            } catch (const Error &e) {  // no room: each sum takes what it needs
+                if (e.code != BEM_ENOMEM) throw;
+            }
+        }
     }
     double *psi = quad_values(m);
     direct_pass(m, SRC_CHARGE, TGT_QUAD_PHI, nullptr, psi);
